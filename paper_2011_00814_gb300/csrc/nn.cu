@@ -575,6 +575,7 @@ cudaError_t conv_dgrad(const ConvArgs& a, cudaStream_t s) {
 }
 
 cudaError_t conv_wgrad(const ConvArgs& a, cudaStream_t s) {
+  if (a.tc && conv_wgrad_tc_supported(a)) return conv_wgrad_tc(a, s);
   const int ks = a.taps == 9 ? 9 : 1;
   dim3 grid((a.cout + BM - 1) / BM, (ks * a.cin + 63) / 64, (a.npix + a.ksplit - 1) / a.ksplit);
   igemm_kernel<2, 64><<<grid, NT, 0, s>>>(a);

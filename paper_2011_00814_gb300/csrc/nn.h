@@ -50,6 +50,8 @@ cudaError_t conv_forward(const ConvArgs& a, cudaStream_t s);
 bool conv_tc_supported(const ConvArgs& a, int mode);
 cudaError_t conv_forward_tc(const ConvArgs& a, cudaStream_t s);
 cudaError_t conv_dgrad_tc(const ConvArgs& a, cudaStream_t s);
+bool conv_wgrad_tc_supported(const ConvArgs& a);
+cudaError_t conv_wgrad_tc(const ConvArgs& a, cudaStream_t s);
 cudaError_t conv_dgrad(const ConvArgs& a, cudaStream_t s);
 cudaError_t conv_wgrad(const ConvArgs& a, cudaStream_t s);
 // dZ = dY silu'(z) and db += sum over pixels of dZ
