@@ -13,6 +13,7 @@
 #include "../../include/gpe2p.h"
 #include "batch.h"
 #include "gpe2p_launch.h"
+#include "step2d.cuh"
 
 using namespace gpe2p;
 
@@ -35,6 +36,11 @@ struct gpe2p_ctx {
   void* Q[3][4] = {};           // three sets of (p, u, v, w): q^n, stage, stage
   void* phi = nullptr;          // phi^{n+1/2}
   void* mu = nullptr;           // mu(phi^{n+1/2})
+  // 2D FP32 problems with the advective RK2 form step phi and mu from one set
+  // into the other with each step (step2d.cuh); elsewhere both sets are one.
+  // phi, mu and phi_lo above and below always name the current set.
+  bool flow_fused = false, ch_fused = false;
+  void *phi2[2] = {}, *mu2[2] = {}, *lo2[2] = {};
   void* phis[2] = {};           // CH stage states
   void* mus = nullptr;          // mu of a CH stage state
   void* acc = nullptr;          // RK4 accumulator
@@ -61,6 +67,7 @@ struct gpe2p_ctx {
   bool initialized = false;
   bool have_graph = false;
   cudaGraphExec_t gexec[2] = {nullptr, nullptr};
+  cudaGraphExec_t gmany = nullptr;  // MANY_STEPS steps from set 0 (2D; built by a long enough gpe2p_advance)
   BatchCtx* batch = nullptr;    // set for a batch of 2D instances
   double* d_dist = nullptr;     // state-distance scratch (allocated on first use)
   double* h_dist = nullptr;
@@ -75,6 +82,14 @@ struct gpe2p_ctx {
   int wait_fault = 0;           // test switch of the 3D kernels' timeout paths (WF_* bits)
   std::string err;
 };
+
+// make set c of the step buffers the current one
+static void set_current(gpe2p_ctx* h, int c) {
+  h->cur = c;
+  h->phi = h->phi2[c];
+  h->mu = h->mu2[c];
+  h->phi_lo = h->lo2[c];
+}
 
 static int fail(gpe2p_ctx* h, int code, const std::string& msg) {
   if (h) h->err = msg;
@@ -311,34 +326,59 @@ static cudaError_t enqueue_step(gpe2p_ctx* h, int cur, ProfHook* hook = nullptr)
   }
   const int s1 = 1 - cur, s2 = 2;
   auto q = [&](int set, int f) { return (real*)h->Q[set][f]; };
-  FlowArgs<real> A{};
-  for (int f = 0; f < 4; ++f) {
-    A.q0[f] = q(cur, f);
-    A.q[f] = q(cur, f);
-    A.out[f] = q(s1, f);
-  }
-  A.phi = (const real*)h->phi;
-  A.mu = (const real*)h->mu;
-  A.a = real(0);
-  A.b = real(1);
-  cudaError_t e = launch_flow_stage<real, DIM>(P, A, 1, h->kchunk, s, &h->flow_maps[cur], h->d_err);
-  if (e != cudaSuccess || (e = mark("flow_stage1")) != cudaSuccess) return e;
-  for (int f = 0; f < 4; ++f) { A.q[f] = q(s1, f); A.out[f] = q(s2, f); }
-  A.a = real(0.75);
-  A.b = real(0.25);
-  if ((e = launch_flow_stage<real, DIM>(P, A, 2, h->kchunk, s, &h->flow_maps[s1], h->d_err)) != cudaSuccess)
-    return e;
-  if ((e = mark("flow_stage2")) != cudaSuccess) return e;
-  for (int f = 0; f < 4; ++f) { A.q[f] = q(s2, f); A.out[f] = q(s1, f); }
-  A.a = real(1.0 / 3.0);
-  A.b = real(2.0 / 3.0);
+  cudaError_t e;
   // advective steps: the last stage also leaves u^n + u^{n+1} per face
   const bool usum = !h->prm.ch_advection;
-  if (usum)
-    for (int a = 0; a < 3; ++a) A.usum[a] = (real*)h->usum[a];
-  if ((e = launch_flow_stage<real, DIM>(P, A, 2, h->kchunk, s, &h->flow_maps[s2], h->d_err)) != cudaSuccess)
-    return e;
-  if ((e = mark("flow_stage3")) != cudaSuccess) return e;
+  if constexpr (DIM == 2 && sizeof(real) == 4) {
+    FlowStepArgs<float> F{};
+    for (int f = 0; f < 3; ++f) {
+      F.q[f] = q(cur, f);
+      F.out[f] = q(s1, f);
+    }
+    F.phi = (const float*)h->phi2[cur];
+    F.mu = (const float*)h->mu2[cur];
+    for (int a = 0; a < 2; ++a) F.usum[a] = usum ? (float*)h->usum[a] : nullptr;
+    if ((e = launch_flow_fused(P, F, s)) != cudaSuccess || (e = mark("flow_step")) != cudaSuccess) return e;
+    if (h->ch_fused) {
+      CHStepArgs<float> G{};
+      G.phi = F.phi;
+      G.mu = F.mu;
+      for (int a = 0; a < 2; ++a) G.usum[a] = (const float*)h->usum[a];
+      G.phi_out = (float*)h->phi2[s1];
+      G.mu_out = (float*)h->mu2[s1];
+      G.lo = (const float*)h->lo2[cur];
+      G.lo_out = (float*)h->lo2[s1];
+      if ((e = launch_ch_fused(P, G, s)) != cudaSuccess) return e;
+      return mark("ch_step");
+    }
+  } else {
+    FlowArgs<real> A{};
+    for (int f = 0; f < 4; ++f) {
+      A.q0[f] = q(cur, f);
+      A.q[f] = q(cur, f);
+      A.out[f] = q(s1, f);
+    }
+    A.phi = (const real*)h->phi;
+    A.mu = (const real*)h->mu;
+    A.a = real(0);
+    A.b = real(1);
+    e = launch_flow_stage<real, DIM>(P, A, 1, h->kchunk, s, &h->flow_maps[cur], h->d_err);
+    if (e != cudaSuccess || (e = mark("flow_stage1")) != cudaSuccess) return e;
+    for (int f = 0; f < 4; ++f) { A.q[f] = q(s1, f); A.out[f] = q(s2, f); }
+    A.a = real(0.75);
+    A.b = real(0.25);
+    if ((e = launch_flow_stage<real, DIM>(P, A, 2, h->kchunk, s, &h->flow_maps[s1], h->d_err)) != cudaSuccess)
+      return e;
+    if ((e = mark("flow_stage2")) != cudaSuccess) return e;
+    for (int f = 0; f < 4; ++f) { A.q[f] = q(s2, f); A.out[f] = q(s1, f); }
+    A.a = real(1.0 / 3.0);
+    A.b = real(2.0 / 3.0);
+    if (usum)
+      for (int a = 0; a < 3; ++a) A.usum[a] = (real*)h->usum[a];
+    if ((e = launch_flow_stage<real, DIM>(P, A, 2, h->kchunk, s, &h->flow_maps[s2], h->d_err)) != cudaSuccess)
+      return e;
+    if ((e = mark("flow_stage3")) != cudaSuccess) return e;
+  }
 
   // Cahn-Hilliard step with the time-centred velocity of Eq. u-center-2d
   CHArgs<real> C{};
@@ -404,20 +444,37 @@ static cudaError_t enqueue(gpe2p_ctx* h, int cur, ProfHook* hook = nullptr) {
   return h->prm.dim == 2 ? enqueue_step<double, 2>(h, cur, hook) : enqueue_step<double, 3>(h, cur, hook);
 }
 
+static void drop_graphs(gpe2p_ctx* h) {
+  for (cudaGraphExec_t* g : {&h->gexec[0], &h->gexec[1], &h->gmany})
+    if (*g) {
+      cudaGraphExecDestroy(*g);
+      *g = nullptr;
+    }
+  h->have_graph = false;
+}
+
+// capture `steps` steps from set c
+static int capture_steps(gpe2p_ctx* h, int c, int steps, cudaGraphExec_t* out) {
+  cudaGraph_t g = nullptr;
+  CK(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeRelaxed), "begin capture");
+  cudaError_t e = cudaSuccess;
+  for (int s = 0; s < steps && e == cudaSuccess; ++s) e = enqueue(h, (c + s) & 1);
+  cudaError_t e2 = cudaStreamEndCapture(h->stream, &g);
+  if (e != cudaSuccess) {
+    if (g) cudaGraphDestroy(g);
+    return cuda_fail(h, e, "enqueue step");
+  }
+  if (e2 != cudaSuccess) return cuda_fail(h, e2, "end capture");
+  e = cudaGraphInstantiate(out, g, 0);
+  cudaGraphDestroy(g);
+  if (e != cudaSuccess) return cuda_fail(h, e, "graph instantiate");
+  return GPE2P_OK;
+}
+
 static int build_graphs(gpe2p_ctx* h) {
   for (int c = 0; c < 2; ++c) {
-    cudaGraph_t g = nullptr;
-    CK(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeRelaxed), "begin capture");
-    cudaError_t e = enqueue(h, c);
-    cudaError_t e2 = cudaStreamEndCapture(h->stream, &g);
-    if (e != cudaSuccess) {
-      if (g) cudaGraphDestroy(g);
-      return cuda_fail(h, e, "enqueue step");
-    }
-    if (e2 != cudaSuccess) return cuda_fail(h, e2, "end capture");
-    e = cudaGraphInstantiate(&h->gexec[c], g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return cuda_fail(h, e, "graph instantiate");
+    const int rc = capture_steps(h, c, 1, &h->gexec[c]);
+    if (rc != GPE2P_OK) return rc;
   }
   h->have_graph = true;
   return GPE2P_OK;
@@ -555,6 +612,13 @@ extern "C" int gpe2p_create(const gpe2p_params* p, void* stream, gpe2p_handle* o
   h->acc = c; c += fb;
   for (int a = 0; a < 3; ++a) { h->uh[a] = c; c += fb; }
   for (int a = 0; a < 3; ++a) { h->usum[a] = c; c += fb; }
+  h->flow_fused = h->prm.dim == 2 && h->esize == 4;
+  h->ch_fused = h->flow_fused && !h->prm.ch_advection && h->prm.ch_scheme == 2;
+  h->phi2[0] = h->phi;
+  h->mu2[0] = h->mu;
+  // the second set lies in the buffers of the per-stage form
+  h->phi2[1] = h->ch_fused ? h->phis[0] : h->phi;
+  h->mu2[1] = h->ch_fused ? h->mus : h->mu;
   h->d_stage = (double*)c; c += stage_b;
   h->d_part = (double*)c; c += part_b;
   h->d_out = (double*)c;
@@ -614,11 +678,14 @@ static int diag_impl(gpe2p_ctx* h, gpe2p_diag* d);
 // are rebuilt at the next step
 static int phi_acc_on(gpe2p_ctx* h) {
   if (h->phi_lo || h->esize != 4) return GPE2P_OK;
-  CK(h, cudaMalloc(&h->phi_lo, field_bytes(h)), "low part of phi");
-  CK(h, cudaMemsetAsync(h->phi_lo, 0, field_bytes(h), h->stream), "low part of phi");
-  for (int c = 0; c < 2; ++c)
-    if (h->gexec[c]) { cudaGraphExecDestroy(h->gexec[c]); h->gexec[c] = nullptr; }
-  h->have_graph = false;
+  const size_t fb = align256(field_bytes(h)), nset = h->ch_fused ? 2 : 1;
+  void* lo = nullptr;
+  CK(h, cudaMalloc(&lo, nset * fb), "low part of phi");
+  h->lo2[0] = lo;
+  h->lo2[1] = (char*)lo + (nset - 1) * fb;
+  set_current(h, h->cur);
+  CK(h, cudaMemsetAsync(lo, 0, nset * fb, h->stream), "low part of phi");
+  drop_graphs(h);
   h->switched_at = h->step;
   return GPE2P_OK;
 }
@@ -694,7 +761,7 @@ extern "C" int gpe2p_init_fields(gpe2p_handle h, const double* phi, const double
   if (h->batch) return fail(h, GPE2P_EINVAL, "a batch handle: use the per-instance calls");
   if (!phi || !u || !v || !p || (h->prm.dim == 3 && !w)) return fail(h, GPE2P_EINVAL, "a required field is NULL");
   CK(h, cudaSetDevice(h->dev), "set device");
-  h->cur = 0;
+  set_current(h, 0);
   // a new state starts with a clear error word (a wait that timed out on the old one)
   CK(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream), "init_fields");
   cudaError_t e = h->esize == 4 ? init_impl<float>(h, phi, u, v, w, p) : init_impl<double>(h, phi, u, v, w, p);
@@ -763,8 +830,22 @@ extern "C" int gpe2p_step(gpe2p_handle h) {
     if (rc != GPE2P_OK) return rc;
   }
   CK(h, cudaGraphLaunch(h->gexec[h->cur], h->stream), "graph launch");
-  h->cur = 1 - h->cur;
+  set_current(h, 1 - h->cur);
   h->step += 1;
+  return GPE2P_OK;
+}
+
+// MANY_STEPS steps (an even number, so that set 0 is current again) by one graph
+constexpr int MANY_STEPS = 16;
+static_assert(MANY_STEPS % 2 == 0, "the graph starts and ends at set 0");
+static int step_many(gpe2p_ctx* h) {
+  CK(h, cudaSetDevice(h->dev), "set device");
+  if (!h->gmany) {
+    const int rc = capture_steps(h, 0, MANY_STEPS, &h->gmany);
+    if (rc != GPE2P_OK) return rc;
+  }
+  CK(h, cudaGraphLaunch(h->gmany, h->stream), "graph launch");
+  h->step += MANY_STEPS;
   return GPE2P_OK;
 }
 
@@ -784,8 +865,19 @@ extern "C" int gpe2p_advance(gpe2p_handle h, long long nsteps, gpe2p_diag* last)
   if (nsteps < 0) return fail(h, GPE2P_EINVAL, "nsteps < 0");
   if (!h->initialized && !h->batch) return fail(h, GPE2P_ESTATE, "gpe2p_advance before gpe2p_init_fields");
   gpe2p_diag d{};
+  // A 2D step is a few launches of some microseconds: a graph of MANY_STEPS of
+  // them costs one graph launch in place of MANY_STEPS.
+  const long long every = h->prm.diag_every > 0 ? h->prm.diag_every : nsteps;
+  const bool many = !h->batch && h->prm.dim == 2 && nsteps >= 2 * MANY_STEPS && every >= 2 * MANY_STEPS;
   for (long long s = 0; s < nsteps; ++s) {
-    int rc = gpe2p_step(h);
+    int rc;
+    const long long left = every - s % every < nsteps - s ? every - s % every : nsteps - s;
+    if (many && h->cur == 0 && left >= MANY_STEPS) {
+      rc = step_many(h);
+      s += MANY_STEPS - 1;
+    } else {
+      rc = gpe2p_step(h);
+    }
     if (rc != GPE2P_OK) return rc;
     if (h->prm.diag_every > 0 && (s + 1) % h->prm.diag_every == 0 && s + 1 < nsteps) {
       rc = any_diag(h, &d);
@@ -823,11 +915,10 @@ extern "C" int gpe2p_set_phi_accumulation(gpe2p_handle h, int mode, double thres
   if (mode == GPE2P_PHI_ACC_COMPENSATED) return phi_acc_on(h);
   if (mode == GPE2P_PHI_ACC_FP32 && h->phi_lo) {
     CK(h, cudaStreamSynchronize(h->stream), "phi accumulation");
-    cudaFree(h->phi_lo);
-    h->phi_lo = nullptr;
-    for (int c = 0; c < 2; ++c)
-      if (h->gexec[c]) { cudaGraphExecDestroy(h->gexec[c]); h->gexec[c] = nullptr; }
-    h->have_graph = false;
+    cudaFree(h->lo2[0]);
+    h->lo2[0] = h->lo2[1] = nullptr;
+    set_current(h, h->cur);
+    drop_graphs(h);
   }
   return GPE2P_OK;
 }
@@ -911,7 +1002,7 @@ static cudaError_t rates_impl(gpe2p_ctx* h) {
   C.phis = (const real*)h->phi;
   C.mus = (const real*)h->mu;
   C.phin = (const real*)h->phi;
-  C.out = (real*)h->phis[0];
+  C.out = (real*)h->phis[1];  // (phis[0] may hold the other set's phi)
   return launch_ch_stage<real, DIM>(P, C, h->prm.iso, h->kchunk_ch, h->stream, &h->ch_maps[0], h->d_err);
 }
 
@@ -925,7 +1016,7 @@ extern "C" int gpe2p_eval_rates(gpe2p_handle h, double* Lp, double* Lu, double* 
   else e = h->prm.dim == 2 ? rates_impl<double, 2>(h) : rates_impl<double, 3>(h);
   if (e != cudaSuccess) return cuda_fail(h, e, "eval_rates");
   double* dst[5] = {Lp, Lu, Lv, h->prm.dim == 3 ? Lw : nullptr, Lphi};
-  const void* src[5] = {h->Q[2][0], h->Q[2][1], h->Q[2][2], h->Q[2][3], h->phis[0]};
+  const void* src[5] = {h->Q[2][0], h->Q[2][1], h->Q[2][2], h->Q[2][3], h->phis[1]};
   for (int f = 0; f < 5; ++f)
     if (dst[f]) CK(h, get_any(h, src[f], dst[f]), "eval_rates copy");
   CK(h, cudaStreamSynchronize(h->stream), "eval_rates sync");
@@ -960,7 +1051,7 @@ extern "C" int gpe2p_profile_steps(gpe2p_handle h, int nsteps, double* ms, int m
     hook.names = nm;
     cudaError_t e = enqueue(h, h->cur, &hook);
     if (e != cudaSuccess) { rc = cuda_fail(h, e, "profile step"); break; }
-    h->cur = 1 - h->cur;
+    set_current(h, 1 - h->cur);
     h->step += 1;
     n = hook.n;
   }
@@ -1015,9 +1106,8 @@ extern "C" void gpe2p_destroy(gpe2p_handle h) {
   if (h->stream) cudaStreamSynchronize(h->stream);
   if (h->d_dist) cudaFree(h->d_dist);
   if (h->h_dist) cudaFreeHost(h->h_dist);
-  if (h->phi_lo) cudaFree(h->phi_lo);
-  for (int c = 0; c < 2; ++c)
-    if (h->gexec[c]) cudaGraphExecDestroy(h->gexec[c]);
+  if (h->lo2[0]) cudaFree(h->lo2[0]);
+  drop_graphs(h);
   if (h->base) cudaFree(h->base);
   if (h->h_out) cudaFreeHost(h->h_out);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
@@ -1107,9 +1197,7 @@ extern "C" int gpe2p_set_fault_injection(gpe2p_handle h, int what, long long val
     } else {
       return fail(h, GPE2P_EINVAL, "a single problem takes GPE2P_FAULT_LOSE_COPY or GPE2P_FAULT_CLEAR");
     }
-    for (int c = 0; c < 2; ++c)
-      if (h->gexec[c]) { cudaGraphExecDestroy(h->gexec[c]); h->gexec[c] = nullptr; }
-    h->have_graph = false;
+    drop_graphs(h);
     return GPE2P_OK;
   }
   if (what == GPE2P_FAULT_LOSE_COPY) return fail(h, GPE2P_EINVAL, "GPE2P_FAULT_LOSE_COPY applies to 3D problems");

@@ -101,6 +101,33 @@ __device__ __forceinline__ real axis_grad_over_r(const T& S, const KParams<real>
   return mul_rn(mul_rn(P.grad_c, sx), fdiv(real(2) * P.inv_dx, real(2 * S.gi + 1)));
 }
 
+// The D2Q9 Laplacian, the (1/r) d/dr of the axisymmetric form and mu of one 2D
+// cell from its three columns: a, b, c point at the rows -1, 0, +1 of the
+// columns -1, 0, +1.  Every kernel that forms mu uses these, so that mu is the
+// same bits wherever it is formed (a run restarted from its fields included).
+template <typename real>
+__device__ __forceinline__ real lap9(const KParams<real>& P, const real* a, const real* b, const real* c) {
+  const real f0 = b[1];
+  real s = mul_rn(P.w2, a[0] - f0);
+  s = fma(P.w1, b[0] - f0, s);
+  s = fma(P.w2, c[0] - f0, s);
+  s = fma(P.w1, a[1] - f0, s);
+  s = fma(P.w1, c[1] - f0, s);
+  s = fma(P.w2, a[2] - f0, s);
+  s = fma(P.w1, b[2] - f0, s);
+  s = fma(P.w2, c[2] - f0, s);
+  return mul_rn(P.lap_c, s);
+}
+template <typename real>
+__device__ __forceinline__ real axis9_over_r(const KParams<real>& P, const real* a, const real* c, int gi) {
+  const real sx = fma(P.w1, c[1] - a[1], mul_rn(P.w2, (c[2] - a[2]) + (c[0] - a[0])));
+  return mul_rn(mul_rn(P.grad_c, sx), fdiv(mul_rn(real(2), P.inv_dx), real(2 * gi + 1)));
+}
+template <typename real>
+__device__ __forceinline__ real chem_pot(const KParams<real>& P, real f, real lap) {
+  return fma(mul_rn(P.a4, f), fma(f, f, real(-1)), -mul_rn(P.kappa, lap));
+}
+
 enum { C_PHI = 0, C_MU = 1, C_UH = 2, C_N = 5 };
 
 // face value of component C on the high face of cell (i,j,k) (the low face of
@@ -340,10 +367,16 @@ __device__ __forceinline__ void mu2d_tile(const KParams<real>& P, const real* __
     S.sm = sm;
     S.c = (2 * ty + r + 1) * SXv + (tx + 1);
     S.gi = i;
-    const real f = S(0, 0, 0, 0);
-    real lap = lap_iso<real, 2, 9>(S, P, 0);
-    if (P.axisym) lap = add_rn(lap, axis_grad_over_r(S, P, 0));  // Eq. chem-pot-axisym
-    out[r] = fma(P.a4 * f, fma(f, f, real(-1)), -(P.kappa * lap));
+    real a[3], b[3], c[3];
+#pragma unroll
+    for (int dy = -1; dy <= 1; ++dy) {
+      a[dy + 1] = S(0, -1, dy, 0);
+      b[dy + 1] = S(0, 0, dy, 0);
+      c[dy + 1] = S(0, 1, dy, 0);
+    }
+    real lap = lap9<real>(P, a, b, c);
+    if (P.axisym) lap = add_rn(lap, axis9_over_r<real>(P, a, c, i));  // Eq. chem-pot-axisym
+    out[r] = chem_pot<real>(P, b[1], lap);
   }
 #pragma unroll
   for (int r = 0; r < 2; ++r) {

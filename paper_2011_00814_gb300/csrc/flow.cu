@@ -366,6 +366,7 @@ cudaError_t launch_flow_stage(const KParams<real>& P, const FlowArgs<real>& A, i
   if (e != cudaSuccess) return e;                                                                         \
   flow2d_kernel<real, M><<<grd, blk, sm, s>>>(P, A);
     if (mode == 0) { GPE2P_FLOW_CASE(0) }
+    else if constexpr (sizeof(real) == 4) { return cudaErrorInvalidValue; }  // FP32 steps in fused passes (step2d.cuh)
     else if (mode == 1) { GPE2P_FLOW_CASE(1) }
     else { GPE2P_FLOW_CASE(2) }
 #undef GPE2P_FLOW_CASE
