@@ -360,6 +360,11 @@ static cudaError_t enqueue_step(gpe2p_ctx* h, int cur, ProfHook* hook = nullptr)
     }
     A.phi = (const real*)h->phi;
     A.mu = (const real*)h->mu;
+    if constexpr (DIM == 2) {
+      // the terms frozen over the stages, in fields the flow of a 2D step leaves free
+      void* z[Z_N] = {h->Q[0][3], h->Q[1][3], h->Q[2][3], h->phis[1], h->acc, h->uh[2], h->usum[2]};
+      for (int k = 0; k < Z_N; ++k) A.z[k] = (real*)z[k];
+    }
     A.a = real(0);
     A.b = real(1);
     e = launch_flow_stage<real, DIM>(P, A, 1, h->kchunk, s, &h->flow_maps[cur], h->d_err);

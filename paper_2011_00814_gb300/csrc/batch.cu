@@ -48,6 +48,7 @@ struct BInst {
   real* phis;      // CH stage state
   real* mus;       // mu of the stage state
   real* uh[2];     // time-centred cell velocity
+  real* z[Z_N];    // FP64: the terms frozen over the flow stages
   real* us[2];     // u^n + u^{n+1} per face (advective form), left by the last flow stage
   int conservative;
 };
@@ -103,14 +104,15 @@ __device__ __forceinline__ void do_sweep(int sw, const BInst<real>& b, const BIt
     A.usum[0] = sums ? b.us[0] : nullptr;
     A.usum[1] = sums ? b.us[1] : nullptr;
     A.usum[2] = nullptr;
+    for (int k = 0; k < Z_N; ++k) A.z[k] = b.z[k];
     if (sw == SW_FLOW1) {
       A.a = real(0);
       A.b = real(1);
-      flow2d_tile<real, 1, TXv, TYv>(b.P, A, it.i0, it.j0, sm);
+      if constexpr (sizeof(real) == 8) flow2d_tile64<1, TXv, TYv, TXv * TYv / 2>(b.P, A, it.i0, it.j0, sm);
     } else {
       A.a = sw == SW_FLOW2 ? real(0.75) : real(1.0 / 3.0);
       A.b = sw == SW_FLOW2 ? real(0.25) : real(2.0 / 3.0);
-      flow2d_tile<real, 2, TXv, TYv>(b.P, A, it.i0, it.j0, sm);
+      if constexpr (sizeof(real) == 8) flow2d_tile64<2, TXv, TYv, TXv * TYv / 2>(b.P, A, it.i0, it.j0, sm);
     }
     return;
   }
@@ -318,7 +320,8 @@ __global__ void __launch_bounds__(TXv* TYv / 2) batch_sweep_kernel(const BInst<r
 
 template <typename real, int TXv, int TYv>
 constexpr size_t batch_smem() {
-  return sizeof(real) * (size_t)F_N * (TXv + 2) * (TYv + 2);  // the largest staged set (flow)
+  // the largest staged set: the FP64 flow stage; in FP32 (conservative instances) the CH stage
+  return sizeof(real) == 8 ? flow64_smem<TXv, TYv>(0) : sizeof(real) * (size_t)C_N * (TXv + 2) * (TYv + 2);
 }
 template <typename real, int TXv, int TYv>
 constexpr size_t persistent_smem() {
@@ -428,7 +431,7 @@ struct BatchCtx {
 };
 
 // field roles inside an instance block
-enum { BF_Q = 0, BF_PHI = 9, BF_MU = 10, BF_PHIS = 11, BF_MUS = 12, BF_UH = 13, BF_US = 15, BF_N = 17 };
+enum { BF_Q = 0, BF_PHI = 9, BF_MU = 10, BF_PHIS = 11, BF_MUS = 12, BF_UH = 13, BF_US = 15, BF_N = 17, BF_Z = 17 };  // FP64: Z_N more
 
 template <typename real>
 static void fill_insts(BatchCtx* b) {
@@ -449,6 +452,7 @@ static void fill_insts(BatchCtx* b) {
     I[k].mu[1] = fld(fused ? BF_MUS : BF_MU);
     I[k].phis = fld(BF_PHIS);
     I[k].mus = fld(BF_MUS);
+    for (int z = 0; z < Z_N; ++z) I[k].z[z] = sizeof(real) == 8 ? fld(BF_Z + z) : nullptr;
     I[k].uh[0] = fld(BF_UH);
     I[k].uh[1] = fld(BF_UH + 1);
     I[k].us[0] = fld(BF_US);
@@ -733,7 +737,7 @@ int batch_create(const gpe2p_params* p, int n, void* stream, BatchCtx** out, std
     if (p[k].ch_advection) b->any_cons = 1;
     const size_t fb = ((size_t)pitch_of(p[k].nx) * p[k].ny * b->esize + 255) / 256 * 256;
     b->field_off.push_back(off);
-    off += fb * BF_N;
+    off += fb * (b->esize == 8 ? BF_N + Z_N : BF_N);
     b->ncell.push_back((long long)p[k].nx * p[k].ny);
     if (b->ncell.back() > maxcell) maxcell = b->ncell.back();
   }

@@ -12,17 +12,41 @@
 namespace gpe2p {
 
 // The single-instance 2D CH stage and mu: one tile per block.
-template <typename real>
-__global__ void __launch_bounds__(NTHR / 2) ch2d_kernel(const KParams<real> P, const CHArgs<real> A) {
+template <typename real, int TXv, int TYv, int CPT>
+__global__ void __launch_bounds__(TXv* TYv / CPT) ch2d_kernel(const __grid_constant__ KParams<real> P,
+                                                          const CHArgs<real> A) {
   extern __shared__ __align__(16) unsigned char smraw2d[];
-  ch2d_tile<real, TX, TY>(P, A, blockIdx.x * TX, blockIdx.y * TY, reinterpret_cast<real*>(smraw2d));
+  ch2d_tile<real, TXv, TYv, CPT>(P, A, blockIdx.x * TXv, blockIdx.y * TYv, reinterpret_cast<real*>(smraw2d));
 }
 
+template <typename real, int TXv, int TYv, int CPT>
+__global__ void __launch_bounds__(TXv* TYv / CPT) mu2d_kernel(const __grid_constant__ KParams<real> P,
+                                                          const real* __restrict__ phi, real* __restrict__ mu) {
+  __shared__ real sm[(TXv + 2) * (TYv + 2)];
+  mu2d_tile<real, TXv, TYv, CPT>(P, phi, mu, blockIdx.x * TXv, blockIdx.y * TYv, sm);
+}
+
+// 32 x 8 tiles of two cells a thread where two fall on every SM, else 8 x 4 of
+// one: a small grid is held back by its busiest SM
 template <typename real>
-__global__ void __launch_bounds__(NTHR / 2) mu2d_kernel(const KParams<real> P, const real* __restrict__ phi,
-                                                    real* __restrict__ mu) {
-  __shared__ real sm[PL];
-  mu2d_tile<real, TX, TY>(P, phi, mu, blockIdx.x * TX, blockIdx.y * TY, sm);
+static bool small2d(const KParams<real>& P) {
+  return (long long)((P.n[0] + TX - 1) / TX) * ((P.n[1] + TY - 1) / TY) < 2 * 152;
+}
+
+template <typename real, int TXv, int TYv, int CPT>
+static cudaError_t ch2d_go(const KParams<real>& P, const CHArgs<real>& A, cudaStream_t s) {
+  constexpr size_t sm = sizeof(real) * (size_t)C_N * (TXv + 2) * (TYv + 2);
+  static_assert(sm <= 48 * 1024, "no opt-in shared memory");
+  const dim3 grd((P.n[0] + TXv - 1) / TXv, (P.n[1] + TYv - 1) / TYv);
+  ch2d_kernel<real, TXv, TYv, CPT><<<grd, TXv * TYv / CPT, sm, s>>>(P, A);
+  return cudaGetLastError();
+}
+
+template <typename real, int TXv, int TYv, int CPT>
+static cudaError_t mu2d_go(const KParams<real>& P, const real* phi, real* mu, cudaStream_t s) {
+  const dim3 grd((P.n[0] + TXv - 1) / TXv, (P.n[1] + TYv - 1) / TYv);
+  mu2d_kernel<real, TXv, TYv, CPT><<<grd, TXv * TYv / CPT, 0, s>>>(P, phi, mu);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -349,11 +373,6 @@ __global__ void center_velocity_kernel(const KParams<real> P, const real* u00, c
   }
 }
 
-template <typename real>
-static size_t ch2d_smem() {
-  return sizeof(real) * (size_t)C_N * PL;
-}
-
 template <typename real, int DIM, int ISO>
 static cudaError_t ch_go(const KParams<real>& P, const CHArgs<real>& A, int kchunk, cudaStream_t s,
                          const Maps<5>* maps, int* err, const Maps<5>* pmaps, const Maps<5>* umaps) {
@@ -396,11 +415,7 @@ static cudaError_t ch_go(const KParams<real>& P, const CHArgs<real>& A, int kchu
       ch3d_kernel<real, ISO, 0, RING, false, false, false><<<grd, blk, sm, s>>>(*maps, *maps, P, A, kchunk, err);
     }
   } else {
-    const size_t sm = ch2d_smem<real>();
-    blk.y = TY / 2;  // two cells per thread
-    e = cudaFuncSetAttribute(ch2d_kernel<real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    ch2d_kernel<real><<<grd, blk, sm, s>>>(P, A);
+    return small2d(P) ? ch2d_go<real, 8, 4, 1>(P, A, s) : ch2d_go<real, TX, TY, 2>(P, A, s);
   }
   return cudaGetLastError();
 }
@@ -435,8 +450,7 @@ static cudaError_t mu_go(const KParams<real>& P, const real* phi, real* mu, int 
     if (e != cudaSuccess) return e;
     mu3d_kernel<real, ISO, RING><<<grd, blk, sm, s>>>(*maps, P, phi, mu, kchunk, err);
   } else {
-    blk.y = TY / 2;  // two cells per thread
-    mu2d_kernel<real><<<grd, blk, 0, s>>>(P, phi, mu);
+    return small2d(P) ? mu2d_go<real, 8, 4, 1>(P, phi, mu, s) : mu2d_go<real, TX, TY, 2>(P, phi, mu, s);
   }
   return cudaGetLastError();
 }

@@ -275,12 +275,12 @@ __device__ __forceinline__ void ch_cell(const T& S, const KParams<real>& P, cons
 }
 
 // One 2D CH stage on the tile of TXv x TYv cells at (i0, j0), by a block of
-// TXv*TYv/2 threads (thread t computes the cells (t % TXv, 2 (t / TXv) + r),
-// r = 0, 1).  sm holds C_N * (TXv+2)*(TYv+2) reals, staged straight from the
+// TXv*TYv/CPT threads (thread t computes the cells (t % TXv, CPT (t / TXv) + r),
+// r < CPT).  sm holds C_N * (TXv+2)*(TYv+2) reals, staged straight from the
 // fields on an interior tile and through the boundary maps at the edges.
 // Stage 1 of the advective form with A.usum set forms the time-centred
 // velocity from the face sums u^n + u^{n+1} the last flow stage left.
-template <typename real, int TXv, int TYv>
+template <typename real, int TXv, int TYv, int CPT = 2>
 __device__ __forceinline__ void ch2d_tile(const KParams<real>& P, const CHArgs<real>& A, int i0, int j0,
                                           real* sm) {
   constexpr int SXv = TXv + 2, SYv = TYv + 2, PLv = SXv * SYv;
@@ -291,16 +291,16 @@ __device__ __forceinline__ void ch2d_tile(const KParams<real>& P, const CHArgs<r
   const bool usum = !cons && A.usum[0] && A.stage == 1;
   const int i = i0 + tx;
   // the per-cell values, loaded first so that their latency overlaps the staging
-  CHPoint<real> c[2] = {};
+  CHPoint<real> c[CPT] = {};
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const int j = j0 + 2 * ty + r;
+  for (int r = 0; r < CPT; ++r) {
+    const int j = j0 + CPT * ty + r;
     if (i < nx && j < ny) {
       if (usum) ch_point_load<real, 2, true>(P, A, i, j, 0, c[r]);
       else ch_point_load<real, 2>(P, A, i, j, 0, c[r]);
     }
   }
-  stage2d<real, TXv, TYv>(P, i0, j0, tile_interior<real, TXv, TYv>(P, i0, j0),
+  stage2d<real, TXv, TYv, TXv * TYv / CPT>(P, i0, j0, tile_interior<real, TXv, TYv>(P, i0, j0),
                           [&](int e, int lx, int ly, long long q) {
     real* b = sm + e;
     if (q >= 0) {
@@ -321,35 +321,35 @@ __device__ __forceinline__ void ch2d_tile(const KParams<real>& P, const CHArgs<r
     }
   });
   __syncthreads();
-  real L[2], ph0[2];
+  real L[CPT], ph0[CPT];
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
+  for (int r = 0; r < CPT; ++r) {
     Tile2<real, SXv, PLv> S;
     S.sm = sm;
-    S.c = (2 * ty + r + 1) * SXv + (tx + 1);
+    S.c = (CPT * ty + r + 1) * SXv + (tx + 1);
     S.gi = i;
     L[r] = ch_rate<real, 2, 9>(S, P, A, c[r]);
     ph0[r] = S(C_PHI, 0, 0, 0);
     if (usum) c[r].pn = ph0[r];  // stage 1: phi^{n+1/2} = phi_s
   }
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const int j = j0 + 2 * ty + r;
+  for (int r = 0; r < CPT; ++r) {
+    const int j = j0 + CPT * ty + r;
     if (i < nx && j < ny) ch_finish<real, 2>(P, A, lin(P, i, j, 0), c[r], L[r], ph0[r]);
   }
   __syncthreads();
 }
 
-// mu of a 2D tile (Eq. chem-pot with the D2Q9 Laplacian) by TXv*TYv/2 threads,
-// two cells each; sm holds (TXv+2)*(TYv+2) reals
-template <typename real, int TXv, int TYv>
+// mu of a 2D tile (Eq. chem-pot with the D2Q9 Laplacian) by TXv*TYv/CPT threads,
+// CPT cells each; sm holds (TXv+2)*(TYv+2) reals
+template <typename real, int TXv, int TYv, int CPT = 2>
 __device__ __forceinline__ void mu2d_tile(const KParams<real>& P, const real* __restrict__ phi,
                                           real* __restrict__ mu, int i0, int j0, real* sm) {
   constexpr int SXv = TXv + 2, PLv = SXv * (TYv + 2);
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
   const int tx = tid % TXv, ty = tid / TXv;
   const int nx = P.n[0], ny = P.n[1];
-  stage2d<real, TXv, TYv>(P, i0, j0, tile_interior<real, TXv, TYv>(P, i0, j0),
+  stage2d<real, TXv, TYv, TXv * TYv / CPT>(P, i0, j0, tile_interior<real, TXv, TYv>(P, i0, j0),
                           [&](int e, int lx, int ly, long long q) {
     if (q >= 0) {
       sm[e] = phi[q];
@@ -360,12 +360,12 @@ __device__ __forceinline__ void mu2d_tile(const KParams<real>& P, const real* __
   });
   __syncthreads();
   const int i = i0 + tx;
-  real out[2];
+  real out[CPT];
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
+  for (int r = 0; r < CPT; ++r) {
     Tile2<real, SXv, PLv> S;
     S.sm = sm;
-    S.c = (2 * ty + r + 1) * SXv + (tx + 1);
+    S.c = (CPT * ty + r + 1) * SXv + (tx + 1);
     S.gi = i;
     real a[3], b[3], c[3];
 #pragma unroll
@@ -379,8 +379,8 @@ __device__ __forceinline__ void mu2d_tile(const KParams<real>& P, const real* __
     out[r] = chem_pot<real>(P, b[1], lap);
   }
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const int j = j0 + 2 * ty + r;
+  for (int r = 0; r < CPT; ++r) {
+    const int j = j0 + CPT * ty + r;
     if (i < nx && j < ny) mu[lin(P, i, j, 0)] = out[r];
   }
   __syncthreads();

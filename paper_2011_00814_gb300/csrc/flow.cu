@@ -5,10 +5,9 @@
 // u-stress-discretization (a)-(d), st-u-discretization, gradp-u-discretization
 // and gradp-u-p-ave-3d, with phi and mu frozen (Sec. 3, after Eq. tvd-rk3).
 //
-// One thread per cell computes the pressure rate at the cell centre and the
-// rate of each velocity component on the cell's low faces (the operators are
-// in flow_ops.cuh).  2D blocks stage one tile with its halo; 3D blocks march
-// along z fed by the TMA plane ring of ring3d.cuh, two cells per thread.
+// The operators are in flow_ops.cuh.  2D blocks stage one tile with its halo;
+// 3D blocks march along z fed by the TMA plane ring of ring3d.cuh, two cells per
+// thread.
 #include "flow_ops.cuh"
 #include "gpe2p_dev.cuh"
 #include "gpe2p_launch.h"
@@ -16,11 +15,43 @@
 
 namespace gpe2p {
 
-// The single-instance 2D flow stage: one tile per block, two cells per thread.
-template <typename real, int MODE>
-__global__ void __launch_bounds__(NTHR / 2) flow2d_kernel(const KParams<real> P, const FlowArgs<real> A) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  flow2d_tile<real, MODE, TX, TY>(P, A, blockIdx.x * TX, blockIdx.y * TY, reinterpret_cast<real*>(smraw));
+// 2D: the FP32 rates (the FP32 step runs in the fused passes of step2d.cuh) and
+// the FP64 stage, one tile per block.
+__global__ void __launch_bounds__(NTHR / 2) rates2d_kernel(const KParams<float> P, const FlowArgs<float> A) {
+  __shared__ float sm2d[F_N * PL];
+  rates2d_tile<float, TX, TY>(P, A, blockIdx.x * TX, blockIdx.y * TY, sm2d);
+}
+
+template <int MODE, int TXv, int TYv, int NT>
+__global__ void __launch_bounds__(NT) flow2d64_kernel(const __grid_constant__ KParams<double> P,
+                                                     const FlowArgs<double> A) {
+  extern __shared__ __align__(16) double sm2d64[];
+  flow2d_tile64<MODE, TXv, TYv, NT>(P, A, blockIdx.x * TXv, blockIdx.y * TYv, sm2d64);
+}
+
+template <int TXv, int TYv, int NT>
+static cudaError_t flow64_go(const KParams<double>& P, const FlowArgs<double>& A, int mode, cudaStream_t s) {
+  static_assert(flow64_smem<TXv, TYv>(0) <= 48 * 1024, "no opt-in shared memory");
+  const size_t sm = flow64_smem<TXv, TYv>(mode);
+  const dim3 grd((P.n[0] + TXv - 1) / TXv, (P.n[1] + TYv - 1) / TYv);
+  if (mode == 0) flow2d64_kernel<0, TXv, TYv, NT><<<grd, NT, sm, s>>>(P, A);
+  else if (mode == 1) flow2d64_kernel<1, TXv, TYv, NT><<<grd, NT, sm, s>>>(P, A);
+  else flow2d64_kernel<2, TXv, TYv, NT><<<grd, NT, sm, s>>>(P, A);
+  return cudaGetLastError();
+}
+
+// The tile of a 2D FP64 stage: 32 x 8 where two tiles fall on every SM, else a
+// smaller one, since a small grid is bound by the FP64 operations of its
+// busiest SM (64 x 64: 16 tiles of 32 x 8 or 128 of 8 x 4).
+// Measured: 20 steps of 64 x 64 with host arrays in and out 1.73 -> 0.80 ms,
+// 50 steps of 128 x 64 4.05 -> 1.56 ms (32 x 8 tiles of FlowOps before).
+static cudaError_t flow64(const KParams<double>& P, const FlowArgs<double>& A, int mode, cudaStream_t s) {
+  auto tiles = [&](int tx, int ty) {
+    return (long long)((P.n[0] + tx - 1) / tx) * ((P.n[1] + ty - 1) / ty);
+  };
+  if (tiles(32, 8) >= 2 * 152) return flow64_go<32, 8, 256>(P, A, mode, s);
+  if (tiles(16, 4) >= 2 * 152) return flow64_go<16, 4, 192>(P, A, mode, s);
+  return flow64_go<8, 4, 96>(P, A, mode, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -326,11 +357,6 @@ __global__ void __launch_bounds__(FLOW_NTHR, FLOW_MINB) flow3d_kernel(const __gr
 template <typename real>
 constexpr int flow_ring() { return GPE2P_FLOW_RING; }
 
-template <typename real>
-static size_t flow2d_smem() {
-  return sizeof(real) * (size_t)F_N * PL;
-}
-
 template <typename real, int DIM>
 cudaError_t launch_flow_stage(const KParams<real>& P, const FlowArgs<real>& A, int mode, int kchunk,
                               cudaStream_t s, const Maps<6>* maps, int* err) {
@@ -358,18 +384,12 @@ cudaError_t launch_flow_stage(const KParams<real>& P, const FlowArgs<real>& A, i
     else if (mode == 1) { GPE2P_FLOW3_CASE(1) }
     else { GPE2P_FLOW3_CASE(2) }
 #undef GPE2P_FLOW3_CASE
+  } else if constexpr (sizeof(real) == 8) {
+    return flow64(P, A, mode, s);
   } else {
-    const size_t sm = flow2d_smem<real>();
+    if (mode != 0) return cudaErrorInvalidValue;  // FP32 steps in fused passes
     blk.y = TY / 2;  // two cells per thread
-#define GPE2P_FLOW_CASE(M)                                                                                \
-  e = cudaFuncSetAttribute(flow2d_kernel<real, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); \
-  if (e != cudaSuccess) return e;                                                                         \
-  flow2d_kernel<real, M><<<grd, blk, sm, s>>>(P, A);
-    if (mode == 0) { GPE2P_FLOW_CASE(0) }
-    else if constexpr (sizeof(real) == 4) { return cudaErrorInvalidValue; }  // FP32 steps in fused passes (step2d.cuh)
-    else if (mode == 1) { GPE2P_FLOW_CASE(1) }
-    else { GPE2P_FLOW_CASE(2) }
-#undef GPE2P_FLOW_CASE
+    rates2d_kernel<<<grd, blk, 0, s>>>(P, A);
   }
   return cudaGetLastError();
 }

@@ -70,7 +70,8 @@ struct FlowArgs {
   const real* phi;     // frozen at t^{n+1/2}
   const real* mu;
   real a, b;
-  real* usum[3];       // 3D mode 2 (last stage): if set, also u0_c + u^{n+1}_c on every face
+  real* usum[3];       // mode 2 (last stage): if set, also u0_c + u^{n+1}_c on every face
+  real* z[7];          // 2D FP64: the terms frozen over the stages, written by mode 1, read by mode 2
 };
 
 // one Cahn-Hilliard stage (Eqs. che, tvd-rk2, rk4) or its rate
