@@ -526,9 +526,10 @@ static bool encode_map(gpe2p_ctx* h, CUtensorMap* m, void* base, int rows, int b
 static int build_maps(gpe2p_ctx* h) {
   bool ok = true;
   for (int s = 0; s < 3; ++s) {
-    for (int f = 0; f < 4; ++f) ok = ok && encode_map(h, &h->flow_maps[s].m[f], h->Q[s][f], FLOW_K3_SY);
-    ok = ok && encode_map(h, &h->flow_maps[s].m[4], h->phi, FLOW_K3_SY);
-    ok = ok && encode_map(h, &h->flow_maps[s].m[5], h->mu, FLOW_K3_SY);
+    const int bx = h->esize == 4 ? FlowGeom<float, FLOW_K3_SY>::BX : FlowGeom<double, FLOW_K3_SY>::BX;
+    for (int f = 0; f < 4; ++f) ok = ok && encode_map(h, &h->flow_maps[s].m[f], h->Q[s][f], FLOW_K3_SY, bx);
+    ok = ok && encode_map(h, &h->flow_maps[s].m[4], h->phi, FLOW_K3_SY, bx);
+    ok = ok && encode_map(h, &h->flow_maps[s].m[5], h->mu, FLOW_K3_SY, bx);
   }
   void* phis[3] = {h->phi, h->phis[0], h->phis[1]};
   void* mus[3] = {h->mu, h->mus, h->mus};
@@ -649,11 +650,10 @@ extern "C" int gpe2p_create(const gpe2p_params* p, void* stream, gpe2p_handle* o
   // SM.  Resident blocks per SM (registers and shared memory, as ncu reports
   // them): flow stage FLOW_MINB, CH stage CH_RESIDENT, mu MU_RESIDENT.
   if (h->prm.dim == 3) {
-    const long long bx = (h->prm.nx + TX - 1) / TX;
     int nsm = 152;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->dev);
-    auto pick = [&](int per_sm, int rows) {
-      const long long bxy = bx * ((h->prm.ny + rows - 1) / rows);
+    auto pick = [&](int per_sm, int cols, int rows) {
+      const long long bxy = (long long)((h->prm.nx + cols - 1) / cols) * ((h->prm.ny + rows - 1) / rows);
       const long long slots = (long long)per_sm * nsm;
       long long best_kc = 4, best = -1;
       for (long long kc = 4; kc <= 64 && kc <= h->prm.nz; ++kc) {
@@ -663,9 +663,9 @@ extern "C" int gpe2p_create(const gpe2p_params* p, void* stream, gpe2p_handle* o
       }
       return (int)(best_kc > h->prm.nz ? h->prm.nz : best_kc);
     };
-    h->kchunk = pick(FLOW_MINB, FLOW_K3_TY);
-    h->kchunk_ch = pick(CH_RESIDENT, CH_K3_TY);
-    h->kchunk_mu = pick(MU_RESIDENT, MU_K3_TY);
+    h->kchunk = pick(h->esize == 4 ? FLOW_MINB : FLOW_MINB64, FLOW_K3_TX, FLOW_K3_TY);
+    h->kchunk_ch = pick(CH_RESIDENT, TX, CH_K3_TY);
+    h->kchunk_mu = pick(MU_RESIDENT, TX, MU_K3_TY);
   } else {
     h->kchunk = h->kchunk_ch = h->kchunk_mu = 1;
   }

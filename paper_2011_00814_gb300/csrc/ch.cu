@@ -63,39 +63,63 @@ struct RawTile {
   }
 };
 
-// wait for plane kk, refill the slot of plane kk - 3 + RING, overwrite the
-// out-of-domain cells of the staged fields with the boundary rules (a block
-// of NT threads staging SYv rows)
-template <typename real, int NRAW, int RING, int SYv, int NT, typename Fix>
+// Wait for plane kk, refill the slot of plane kk - 3 + RING, set the ghost cells
+// of the staged fields (a block of NT threads staging SYv rows): those of a tile
+// on the boundary, all of a plane beyond a periodic z side.  kinds[f], src[f]:
+// the field's ghost rule and its global array.
+template <typename real, int NRAW>
+struct RingFields {
+  int kind[NRAW];
+  const real* src[NRAW];
+};
+template <typename real, int NRAW, int RING, int SYv, int NT>
 __device__ __forceinline__ bool ring_acquire(Ring<real, NRAW, RING, SYv>& R, const KParams<real>& P,
                                              const CUtensorMap* maps, int kk, bool refill, bool edge_tile,
-                                             Fix fix) {
+                                             const RingFields<real, NRAW>& F) {
   using G = RingGeom<real, SYv>;
   if (!R.wait(kk)) return false;
   const int tid = threadIdx.y * TX + threadIdx.x;
-  if (refill && tid == 0) R.refill(P, maps, kk);
+  if (refill) R.refill(P, maps, kk);
   const bool ghost_plane = kk < 0 || kk >= P.n[2];
-  if (ghost_plane || edge_tile) {
-    // a full tile can reach outside the domain only on the staged region's
-    // perimeter; a tile that overhangs the domain end has its ghost column or
-    // row inside the region, so it and a ghost plane are scanned in full
-    const bool full = ghost_plane || R.i0 + TX > P.n[0] || R.j0 + (SYv - 2) > P.n[1];
-    const int ncell = full ? SX * SYv : perim<SYv>();
-    for (int q = tid; q < ncell; q += NT) {
-      int lx, ly;
-      if (full) { ly = q / SX; lx = q - ly * SX; }
-      else perim_cell<SYv>(q, lx, ly);
-      const int gi = R.i0 - 1 + lx, gj = R.j0 - 1 + ly;
-      if (ghost_plane || gi < 0 || gi >= P.n[0] || gj < 0 || gj >= P.n[1]) {
-        const int ci = clampi(gi, -1, P.n[0]), cj = clampi(gj, -1, P.n[1]);
+  if (ghost_plane ? P.bc[2] == BC_PERIODIC : edge_tile) {
+    if (ghost_plane) {
+      for (int q = tid; q < SX * SYv; q += NT) {
+        const int ly = q / SX, lx = q - ly * SX;
+        const int ci = clampi(R.i0 - 1 + lx, -1, P.n[0]), cj = clampi(R.j0 - 1 + ly, -1, P.n[1]);
         const int e = G::at(lx, ly);
 #pragma unroll
-        for (int f = 0; f < NRAW; ++f) R.plane(kk, f)[e] = fix(f, ci, cj, kk);
+        for (int f = 0; f < NRAW; ++f) R.plane(kk, f)[e] = ld_kind(F.kind[f], F.src[f], P, ci, cj, kk);
+      }
+    } else {
+      static_assert(ghost_count<SYv>() <= NT, "a ghost cell per thread");
+      int lx, ly;
+      if (tid < ghost_count<SYv>() && ghost_cell<SYv>(P, R.i0, R.j0, tid, lx, ly)) {
+        const int e = G::at(lx, ly);
+#pragma unroll
+        for (int f = 0; f < NRAW; ++f) {
+          real* pl = R.plane(kk, f);
+          pl[e] = ghost_value<G>(F.kind[f], pl, F.src[f], P, R.i0, R.j0, R.i0 - 1 + lx, R.j0 - 1 + ly, kk);
+        }
       }
     }
     fence_proxy_async_smem();
   }
   return true;
+}
+
+// the plane kk beyond a z wall from the plane next to it, after a barrier that
+// follows that plane's ghost writes
+template <typename real, int NRAW, int RING, int SYv, int NT>
+__device__ __forceinline__ void ring_zwall(Ring<real, NRAW, RING, SYv>& R, const KParams<real>& P, int kk) {
+  using G = RingGeom<real, SYv>;
+  const int from = kk < 0 ? 0 : P.n[2] - 1;
+  for (int q = threadIdx.y * TX + threadIdx.x; q < G::BX * SYv; q += NT)
+#pragma unroll
+    for (int f = 0; f < NRAW; ++f) {
+      const real v = R.plane(from, f)[q];
+      R.plane(kk, f)[q] = f == C_UH + 2 ? -v : v;  // uhat_z is odd, the rest even
+    }
+  fence_proxy_async_smem();
 }
 
 // One block: a TX x CH_K3_TY column of cells over the planes [kbeg, kend);
@@ -136,21 +160,27 @@ __global__ void __launch_bounds__(CH_NTHR) ch3d_kernel(const __grid_constant__ M
   bool act[CH_CPT];
 #pragma unroll
   for (int r = 0; r < CH_CPT; ++r) act[r] = i < nx && ja + r < ny;
-  auto fix = [&](int f, int ci, int cj, int kk) -> real {
-    switch (f) {
-      case C_PHI: return ld_cen(A.phis, P, ci, cj, kk);
-      case C_MU: return ld_cen(A.mus, P, ci, cj, kk);
-      case C_UH + 0: return ld_cvec<0>(A.uh[0], P, ci, cj, kk);
-      case C_UH + 1: return ld_cvec<1>(A.uh[1], P, ci, cj, kk);
-      default: return ld_cvec<2>(A.uh[2], P, ci, cj, kk);
+  RingFields<real, NRAW> F;
+  F.kind[C_PHI] = F.kind[C_MU] = K_CEN;
+  F.src[C_PHI] = A.phis;
+  F.src[C_MU] = A.mus;
+  if constexpr (CONS) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      F.kind[C_UH + a] = K_CVEC0 + a;
+      F.src[C_UH + a] = A.uh[a];
     }
-  };
+  }
+  const bool zwalls = P.bc[2] != BC_PERIODIC;
   // point planes (PTS): two slots after the ring, their barriers after the ring's
   const int tid = ty * TX + tx;
   uint64_t* pbar = R.bar + 8;
   real* pts = R.raw + (size_t)RING * NRAW * G::PE;
   const bool need_acc = (A.scheme == 4 && A.stage >= 2) || (A.phi_lo && A.scheme == 2 && A.stage == 2);
-  int pissued = kbeg - 1;  // thread 0: last point plane issued
+  // (issued by another warp than the ring's refills, so that neither holds the
+  // block at the next barrier for both)
+  const bool pissuer = tx == 0 && ty == 1;
+  int pissued = kbeg - 1;  // issuer: last point plane issued
   auto pissue = [&](int kk) {
     if (kk >= kend) return;
     uint64_t* b = &pbar[(kk - kbeg) & 1];
@@ -163,13 +193,13 @@ __global__ void __launch_bounds__(CH_NTHR) ch3d_kernel(const __grid_constant__ M
   };
   // after a ring timeout: let this block's point copies in flight land
   auto pdrain = [&](int from) {
-    if (PTS && tid == 0)
+    if (PTS && pissuer)
       for (int kk = from; kk <= pissued; ++kk)
         mbar_wait_bounded(&pbar[(kk - kbeg) & 1], ((kk - kbeg) >> 1) & 1, WAIT_CYCLES / 2);
   };
   // UPTS: the face-sum point planes kbeg .. klast
   const int klast = min(kend, P.n[2] - 1);
-  int uissued = kbeg - 1;  // thread 0: last face-sum plane issued
+  int uissued = kbeg - 1;  // issuer: last face-sum plane issued
   auto uslot = [&](int kk) { return (kk - kbeg) % 3; };
   auto upar = [&](int kk) { return (uint32_t)(((kk - kbeg) / 3) & 1); };
   auto uissue = [&](int kk) {
@@ -183,22 +213,24 @@ __global__ void __launch_bounds__(CH_NTHR) ch3d_kernel(const __grid_constant__ M
     uissued = kk;
   };
   auto udrain = [&](int from) {
-    if (UPTS && tid == 0)
+    if (UPTS && pissuer)
       for (int kk = from; kk <= uissued; ++kk) mbar_wait_bounded(&pbar[uslot(kk)], upar(kk), WAIT_CYCLES / 2);
   };
   if ((PTS || UPTS) && tid == 0) {
-    mbar_init(&pbar[0], 1);
-    mbar_init(&pbar[1], 1);
-    mbar_init(&pbar[2], 1);
+    for (int b = 0; b < 3; ++b) mbar_init(&pbar[b], 1);
   }
   R.start(P, maps.m, kbeg, kend, i0, j0, (P.wait_fault & WF_CH_RING) != 0);
-  if (PTS && tid == 0) pissue(kbeg);
-  if (UPTS && tid == 0) {
+  if (PTS && pissuer) pissue(kbeg);
+  if (UPTS && pissuer) {
     uissue(kbeg);
     uissue(kbeg + 1);
   }
-  if (!ring_acquire<real, NRAW, RING, CH_K3_SY, CH_NTHR>(R, P, maps.m, kbeg - 1, false, edge_tile, fix)) { R.fail(err, kbeg - 1); pdrain(kbeg); udrain(kbeg); return; }
-  if (!ring_acquire<real, NRAW, RING, CH_K3_SY, CH_NTHR>(R, P, maps.m, kbeg, false, edge_tile, fix)) { R.fail(err, kbeg); pdrain(kbeg); udrain(kbeg); return; }
+  if (!ring_acquire<real, NRAW, RING, CH_K3_SY, CH_NTHR>(R, P, maps.m, kbeg - 1, false, edge_tile, F)) { R.fail(err, kbeg - 1); pdrain(kbeg); udrain(kbeg); return; }
+  if (!ring_acquire<real, NRAW, RING, CH_K3_SY, CH_NTHR>(R, P, maps.m, kbeg, false, edge_tile, F)) { R.fail(err, kbeg); pdrain(kbeg); udrain(kbeg); return; }
+  if (kbeg == 0 && zwalls) {
+    if (edge_tile) __syncthreads();  // plane 0's ghosts
+    ring_zwall<real, NRAW, RING, CH_K3_SY, CH_NTHR>(R, P, -1);
+  }
   bool pfail = false;  // a point-plane wait of this thread gave up
   // test switch: the first point-plane wait completes, then reports a timeout
   const bool plose = (P.wait_fault & WF_CH_POINTS) != 0;
@@ -219,10 +251,10 @@ __global__ void __launch_bounds__(CH_NTHR) ch3d_kernel(const __grid_constant__ M
       for (int r = 0; r < CH_CPT; ++r)
         if (act[r]) ch_point_load<real, 3, USUM>(P, A, i, ja + r, k, c[r]);
     }
-    if (!ring_acquire<real, NRAW, RING, CH_K3_SY, CH_NTHR>(R, P, maps.m, k + 1, true, edge_tile, fix)) { R.fail(err, k + 1); pdrain(k); udrain(k + 1); return; }
+    if (!ring_acquire<real, NRAW, RING, CH_K3_SY, CH_NTHR>(R, P, maps.m, k + 1, true, edge_tile, F)) { R.fail(err, k + 1); pdrain(k); udrain(k + 1); return; }
     if (UPTS) {
       // every thread is past plane k - 1: its slot takes plane k + 2
-      if (tid == 0) uissue(k + 2);
+      if (pissuer) uissue(k + 2);
       if (k + 1 <= klast && !mbar_wait_bounded(&pbar[uslot(k + 1)], upar(k + 1), WAIT_CYCLES)) {
         atomicExch(err, ERR_TMA_TIMEOUT);
         pfail = true;
@@ -252,7 +284,7 @@ __global__ void __launch_bounds__(CH_NTHR) ch3d_kernel(const __grid_constant__ M
     }
     if (PTS) {
       // every thread is past plane k - 1: its slot takes plane k + 1
-      if (tid == 0) pissue(k + 1);
+      if (pissuer) pissue(k + 1);
       if (!mbar_wait_bounded(&pbar[(k - kbeg) & 1], ((k - kbeg) >> 1) & 1, WAIT_CYCLES) || (plose && k == kbeg)) {
         atomicExch(err, ERR_TMA_TIMEOUT);
         pfail = true;
@@ -266,7 +298,9 @@ __global__ void __launch_bounds__(CH_NTHR) ch3d_kernel(const __grid_constant__ M
         c[r].acc = pp[4 * CP_PT + r * TX];
       }
     }
-    if (edge_tile || k + 1 >= P.n[2]) __syncthreads();  // out-of-domain writes seen by all
+    // (plane nz - 1 was set and read in the last turn)
+    if (k + 1 == P.n[2] && zwalls) ring_zwall<real, NRAW, RING, CH_K3_SY, CH_NTHR>(R, P, k + 1);
+    if (edge_tile || k + 1 >= P.n[2]) __syncthreads();  // ghost writes seen by all
     real L[CH_CPT], ph0[CH_CPT];
 #pragma unroll
     for (int r = 0; r < CH_CPT; ++r) {
@@ -283,10 +317,10 @@ __global__ void __launch_bounds__(CH_NTHR) ch3d_kernel(const __grid_constant__ M
     for (int r = 0; r < CH_CPT; ++r)
       if (act[r]) ch_finish<real, 3>(P, A, lin(P, i, ja + r, k), c[r], L[r], ph0[r]);
   }
-  // a point-plane wait of thread 0 gave up (the error word is set): let the
+  // a point-plane wait of the issuer gave up (the error word is set): let the
   // last copies into each slot land before the block exits; a phase that
   // never completed also holds the bytes of the copies issued after it
-  if ((PTS || UPTS) && tid == 0 && pfail) {
+  if ((PTS || UPTS) && pissuer && pfail) {
     if (PTS)
       for (int kk = pissued; kk >= kbeg && kk > pissued - 2; --kk)
         mbar_wait_bounded(&pbar[(kk - kbeg) & 1], ((kk - kbeg) >> 1) & 1, WAIT_CYCLES / 2);
@@ -317,15 +351,21 @@ __global__ void __launch_bounds__(MU_NTHR) mu3d_kernel(const __grid_constant__ M
   bool act[MU_CPT];
 #pragma unroll
   for (int r = 0; r < MU_CPT; ++r) act[r] = i < nx && ja + r < ny;
-  auto fix = [&](int, int ci, int cj, int kk) -> real { return ld_cen(phi, P, ci, cj, kk); };
+  const RingFields<real, 1> F = {{K_CEN}, {phi}};
+  const bool zwalls = P.bc[2] != BC_PERIODIC;
   R.start(P, maps.m, kbeg, kend, i0, j0, (P.wait_fault & WF_MU_RING) != 0);
-  if (!ring_acquire<real, 1, RING, MU_K3_SY, MU_NTHR>(R, P, maps.m, kbeg - 1, false, edge_tile, fix)) { R.fail(err, kbeg - 1); return; }
-  if (!ring_acquire<real, 1, RING, MU_K3_SY, MU_NTHR>(R, P, maps.m, kbeg, false, edge_tile, fix)) { R.fail(err, kbeg); return; }
+  if (!ring_acquire<real, 1, RING, MU_K3_SY, MU_NTHR>(R, P, maps.m, kbeg - 1, false, edge_tile, F)) { R.fail(err, kbeg - 1); return; }
+  if (!ring_acquire<real, 1, RING, MU_K3_SY, MU_NTHR>(R, P, maps.m, kbeg, false, edge_tile, F)) { R.fail(err, kbeg); return; }
+  if (kbeg == 0 && zwalls) {
+    if (edge_tile) __syncthreads();  // plane 0's ghosts
+    ring_zwall<real, 1, RING, MU_K3_SY, MU_NTHR>(R, P, -1);
+  }
   const real* smr = reinterpret_cast<const real*>(smraw);
   const int raw0 = (int)(R.raw - smr), cell0 = G::at(tx + 1, MU_CPT * ty + 1);
   for (int k = kbeg; k < kend; ++k) {
-    if (!ring_acquire<real, 1, RING, MU_K3_SY, MU_NTHR>(R, P, maps.m, k + 1, true, edge_tile, fix)) { R.fail(err, k + 1); return; }
-    if (edge_tile || k + 1 >= P.n[2]) __syncthreads();  // out-of-domain writes seen by all
+    if (!ring_acquire<real, 1, RING, MU_K3_SY, MU_NTHR>(R, P, maps.m, k + 1, true, edge_tile, F)) { R.fail(err, k + 1); return; }
+    if (k + 1 == P.n[2] && zwalls) ring_zwall<real, 1, RING, MU_K3_SY, MU_NTHR>(R, P, k + 1);
+    if (edge_tile || k + 1 >= P.n[2]) __syncthreads();  // ghost writes seen by all
     real m[MU_CPT];
 #pragma unroll
     for (int r = 0; r < MU_CPT; ++r) {

@@ -58,199 +58,96 @@ static cudaError_t flow64(const KParams<double>& P, const FlowArgs<double>& A, i
 // 3D: the same stage fed by the TMA plane ring of ring3d.cuh
 // ---------------------------------------------------------------------------
 
-// fields staged per plane; rho, eta and nu are formed from phi where they are read
+// fields staged per plane; rho, eta and nu are formed from phi
 enum { R_P = 0, R_U = 1, R_V = 2, R_W = 3, R_PHI = 4, R_MU = 5, NRAW_FLOW = 6 };
 
-template <typename real, int PAVG_>
-struct RingTile {
-  static constexpr int PAVG = PAVG_;
-  using G = RingGeom<real, FLOW_K3_SY>;
-  const real* sm;           // the block's shared memory
-  const KParams<real>* P;
-  int r[3];                 // index of the thread's cell in raw field 0 of planes k-1, k, k+1
-  __device__ __forceinline__ real raw(int f, int o, int dz) const { return sm[r[dz + 1] + f * G::PE + o]; }
-  __device__ __forceinline__ real operator()(int f, int dx, int dy, int dz) const {
-    const int o = dy * G::BX + dx;
-    switch (f) {
-      case F_P: return raw(R_P, o, dz);
-      case F_U: return raw(R_U, o, dz);
-      case F_V: return raw(R_V, o, dz);
-      case F_W: return raw(R_W, o, dz);
-      case F_PHI: return raw(R_PHI, o, dz);
-      case F_MU: return raw(R_MU, o, dz);
-      case F_RHO: return rho_of(*P, raw(R_PHI, o, dz));
-      case F_ETA: return eta_of(*P, raw(R_PHI, o, dz));
-      default: {  // F_NU
-        const real phi = raw(R_PHI, o, dz);
-        return fdiv(eta_of(*P, phi), rho_of(*P, phi));
-      }
-    }
-  }
+// a / rho: the approximate reciprocal of a normal number needs none of the
+// range handling of the general quotient (five instructions of seven); FP64: the
+// IEEE quotient
+__device__ __forceinline__ float quot_rho(float a, float rho) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(rho));
+  return a * r;
+}
+__device__ __forceinline__ double quot_rho(double a, double rho) { return a / rho; }
+
+// Material and viscosity sums of one plane at the thread's column: rows -1 .. R.
+template <typename real, int R>
+struct FlowMat {
+  real eta[R + 2], nu[R + 2];  // eta / dx^2 and nu / dx^2, rows -1 .. R
+  real rho[R + 1];             // rows -1 .. R-1
+  real sx[R + 2];              // eta(i) + eta(i-1), rows -1 .. R
+  real sy[R + 1];              // eta(j) + eta(j-1), rows 0 .. R
 };
 
-// The -z side terms of a cell's 3D rates are what the same thread formed on
-// the +z side of the cell below, one plane earlier: the stresses on the x-z
-// and y-z edges between the two planes (the u and v faces' -z edge terms, and
-// the w face's -x and -y edge terms, are their negatives), the averaged
-// pressure and the divergence of the cell below (the w face's gradient and
-// bulk terms), and the flux nu (p_k - p_{k-1}) of the pressure diffusion.
-// The block marches along z, so these are carried in registers.
-template <typename real>
-struct ZCarry {
-  real tau_xz, tau_yz;  // 4 eta_edge x (du/dz + dw/dx) and (dv/dz + dw/dy), times dx, on the +z edges
-  real psum2;           // 36 x the pressure averaged over the x-y plane (Eq. gradp-u-p-ave-3d)
-  real div;             // dx div u
-  real pflux;           // (nu + nu(+z)) (p(+z) - p)
+// The terms of the faces and edges between a plane and the one above it, and the
+// plane's x-y averaged pressure.  The block marches along z, so the values
+// formed above one plane are those below the next and stay in registers.
+template <typename real, int R>
+struct FlowZ {
+  real txz[R];      // 4 eta_edge/dx^2 (du/dz + dw/dx) dx on the x-z edges, rows 0 .. R-1
+  real tyz[R + 1];  // the y-z edges, rows 0 .. R
+  real tz[R];       // normal stress of the plane's cells along z
+  real fz[R];       // (nu + nu(+z)) (p(+z) - p)
+  real xy[R];       // 36 x the pressure averaged over x and y
+  real rho[R];
 };
 
-// FlowOps with the -z side terms taken from the carry of the plane below and
-// the +z side terms returned for the plane above (3D ring tiles only)
-template <typename real, typename T>
-struct FlowOpsZ : FlowOps<real, 3, T> {
-  using B = FlowOps<real, 3, T>;
-
-  // the +z side terms of the cell (planes 0 and +1 only); d0 = dx div u of the cell
-  __device__ __forceinline__ static void plus_z(const T& S, const KParams<real>& P, real d0, ZCarry<real>& o) {
-    real e4p, e4m;
-    B::template edge_eta4<0>(S, 2, e4p, e4m);
-    o.tau_xz = e4p * ((S(F_U, 0, 0, 1) - S(F_U, 0, 0, 0)) + (S(F_W, 0, 0, 1) - S(F_W, -1, 0, 1)));
-    B::template edge_eta4<1>(S, 2, e4p, e4m);
-    o.tau_yz = e4p * ((S(F_V, 0, 0, 1) - S(F_V, 0, 0, 0)) + (S(F_W, 0, 0, 1) - S(F_W, 0, -1, 1)));
-    o.psum2 = B::averaged(P) ? B::template psum<2>(S, 0, 0, 0) : real(0);
-    o.div = d0;
-    o.pflux = (S(F_NU, 0, 0, 0) + S(F_NU, 0, 0, 1)) * (S(F_P, 0, 0, 1) - S(F_P, 0, 0, 0));
-  }
-
-  // the pressure rate with the -z flux from the carry
-  __device__ __forceinline__ static real rate_p(const T& S, const KParams<real>& P, real d0, const ZCarry<real>& in,
-                                                const ZCarry<real>& out) {
-    real diff = out.pflux - in.pflux;
-    const real nu0 = S(F_NU, 0, 0, 0), p0 = S(F_P, 0, 0, 0);
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-      const int ex = a == 0, ey = a == 1;
-      diff = fma(nu0 + S(F_NU, ex, ey, 0), S(F_P, ex, ey, 0) - p0, diff);
-      diff = fma(nu0 + S(F_NU, -ex, -ey, 0), S(F_P, -ex, -ey, 0) - p0, diff);
-    }
-    return fma(diff, real(0.5) * P.inv_dx2, -(S(F_RHO, 0, 0, 0) * P.cs2 * mul_rn(d0, P.inv_dx)));
-  }
-
-  // the velocity rate of component C with its z-side (C = 0, 1) or x- and
-  // y-side (C = 2) edge terms below the cell, and the w face's averaged
-  // pressure and divergence below, from the carry
-  template <int C>
-  __device__ __forceinline__ static real rate_vel(const T& S, const KParams<real>& P, real d0,
-                                                  const ZCarry<real>& in, const ZCarry<real>& out) {
-    constexpr int cx = C == 0, cy = C == 1, cz = C == 2;
-    const int FC = F_U + C;
-    const real rb2 = S(F_RHO, -cx, -cy, -cz) + S(F_RHO, 0, 0, 0);
-    real gradp;
-    if (B::averaged(P)) {
-      const real pm = C == 2 ? in.psum2 : B::template psum<C>(S, -cx, -cy, -cz);
-      const real p0 = C == 2 ? out.psum2 : B::template psum<C>(S, 0, 0, 0);
-      gradp = (p0 - pm) * (P.inv_dx * real(1.0 / 36.0));
-    } else {
-      gradp = (S(F_P, 0, 0, 0) - S(F_P, -cx, -cy, -cz)) * P.inv_dx;
-    }
-    const real uc0 = S(FC, 0, 0, 0);
-    const real tcc = fma(S(F_ETA, -cx, -cy, -cz), S(FC, -cx, -cy, -cz) - uc0,
-                         mul_rn(S(F_ETA, 0, 0, 0), S(FC, cx, cy, cz) - uc0));
-    real edge = real(0), conv4 = real(0);
-#pragma unroll
-    for (int t = 0; t < 3; ++t) {
-      if (t == C) continue;
-      const int tx = t == 0, ty = t == 1, tz = t == 2;
-      const int FT = F_U + t;
-      const real ucp = S(FC, tx, ty, tz), ucm = S(FC, -tx, -ty, -tz);
-      const real ut0 = S(FT, 0, 0, 0), utc = S(FT, -cx, -cy, -cz);
-      const real utp = S(FT, tx, ty, tz), utpc = S(FT, tx - cx, ty - cy, tz - cz);
-      if (t == 2) {
-        // the x-z or y-z edges above and below the u or v face
-        edge += (C == 0 ? out.tau_xz : out.tau_yz) - (C == 0 ? in.tau_xz : in.tau_yz);
-      } else if (C == 2) {
-        // the w face: the edge on its -t side lies between the planes, below the cell
-        real e4p, e4m;
-        B::template edge_eta4<C>(S, t, e4p, e4m);
-        edge = fma(e4p, (ucp - uc0) + (utp - utpc), edge);
-        edge -= t == 0 ? in.tau_xz : in.tau_yz;
-      } else {
-        real e4p, e4m;
-        B::template edge_eta4<C>(S, t, e4p, e4m);
-        edge = fma(e4p, (ucp - uc0) + (utp - utpc), edge);
-        edge = fma(e4m, (ucm - uc0) + (utc - ut0), edge);
-      }
-      conv4 = fma((ut0 + utc) + (utp + utpc), ucp - ucm, conv4);
-    }
-    real visc = fma(real(2), tcc, mul_rn(real(0.25), edge));
-    if (P.bulk) {
-      const real dm = C == 2 ? in.div : B::divsum(S, P, -cx, -cy, -cz);
-      visc = fma(S(F_ETA, 0, 0, 0), d0, visc);
-      visc = fma(-S(F_ETA, -cx, -cy, -cz), dm, visc);
-    }
-    const real st = -P.sigma * (S(F_PHI, 0, 0, 0) + S(F_PHI, -cx, -cy, -cz)) *
-                    (S(F_MU, 0, 0, 0) - S(F_MU, -cx, -cy, -cz));
-    const real grav = fma(real(0.5), rb2, -P.rho_ref);
-    real force = fma(visc, P.inv_dx2, -gradp);
-    force = fma(st, P.inv_2dx, force);
-    force = fma(grav, P.g[C], force);
-    const real conv = fma(uc0, S(FC, cx, cy, cz) - S(FC, -cx, -cy, -cz), mul_rn(real(0.25), conv4));
-    return fma(-conv, P.inv_2dx, fdiv(real(2) * force, rb2));
-  }
-};
-
-// One block: a TX x FLOW_K3_TY column of cells over the planes [kbeg, kend);
-// thread (tx, ty) computes the cells (i0 + tx, j0 + 2 ty + r), r = 0, 1.  The
-// two cells share most of their stencil, so the loads and sub-expressions
-// they have in common are formed once.
-// resident blocks per SM the 3D flow stage is compiled for (FLOW_MINB: up to
-// 128 registers, no spills; three blocks of 256 threads cap them at 80 with
-// spills and measured slower, 5.61 against 4.88 ms per step of the
-// 256x256x512 bubble)
-
+// One block: FLOW_K3_TX x FLOW_K3_TY cells of a column over the planes
+// [kbeg, kend).  Lane = staged column (30 of the 32 are the block's own);
+// each thread takes R = 2 adjacent rows.
+//
+// What bounds it: instruction issue, not HBM.  So every term that two
+// cells share is formed once: the normal stresses, corner stresses, diffusive
+// fluxes and averaged pressures of a column go to its left or right
+// neighbour by a shuffle, to the row above in registers (the two rows beyond
+// the thread's own are formed twice), and to the plane above in registers
+// (FlowZ); averages are taken axis by axis.  The price is two idle
+// lanes of 32.  Stage 2 of 128 x 128 x 256 (ncu): 105 us, 218 floating-point
+// instructions a cell; 121 us and 365 with each thread forming all terms of its
+// two cells.
+// FLOW_MINB blocks of four warps per SM: 128 registers (FP64: two blocks, which
+// its ALU rate keeps busy).
 template <typename real, int MODE, int RING, int PAVG>
-__global__ void __launch_bounds__(FLOW_NTHR, FLOW_MINB) flow3d_kernel(const __grid_constant__ Maps<NRAW_FLOW> maps,
-                                                      const __grid_constant__ KParams<real> P,
-                                                      const FlowArgs<real> A, const int kchunk, int* err) {
-  constexpr int SYv = FLOW_K3_SY;
-  using G = RingGeom<real, SYv>;
+__global__ void __launch_bounds__(FLOW_NTHR, sizeof(real) == 8 ? FLOW_MINB64 : FLOW_MINB)
+    flow3d_kernel(const __grid_constant__ Maps<NRAW_FLOW> maps, const __grid_constant__ KParams<real> P,
+                  const FlowArgs<real> A, const int kchunk, int* err) {
+  constexpr int SYv = FLOW_K3_SY, R = 2;
+  using G = FlowGeom<real, SYv>;
+  constexpr unsigned FULL = 0xffffffffu;
   extern __shared__ __align__(128) unsigned char smraw[];
-  Ring<real, NRAW_FLOW, RING, SYv> R;
+  Ring<real, NRAW_FLOW, RING, SYv, G, FLOW_TY> Rg;
   unsigned char* sbase = smem_base128(smraw);
-  R.bar = reinterpret_cast<uint64_t*>(sbase);
-  R.raw = reinterpret_cast<real*>(sbase + 128);
+  Rg.bar = reinterpret_cast<uint64_t*>(sbase);
+  Rg.raw = reinterpret_cast<real*>(sbase + 128);
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
-  const int i0 = blockIdx.x * TX, j0 = blockIdx.y * FLOW_K3_TY;
+  const int i0 = blockIdx.x * FLOW_K3_TX, j0 = blockIdx.y * FLOW_K3_TY;
   const int kbeg = blockIdx.z * kchunk;
   const int kend = min(kbeg + kchunk, P.n[2]);
   const int nx = P.n[0], ny = P.n[1], nz = P.n[2];
-  const bool edge_tile = i0 == 0 || i0 + TX + 1 > nx || j0 == 0 || j0 + FLOW_K3_TY + 1 > ny;
-  const bool ragged = i0 + TX > nx || j0 + FLOW_K3_TY > ny;
-  const int i = i0 + tx, ja = j0 + 2 * ty;
-  const bool act[2] = {i < nx && ja < ny, i < nx && ja + 1 < ny};
+  const bool edge_tile = i0 == 0 || i0 + 31 > nx || j0 == 0 || j0 + FLOW_K3_TY + 1 > ny;
+  const int i = i0 - 1 + tx, ja = j0 + 2 * ty;
+  const bool own = tx >= 1 && tx <= FLOW_K3_TX && i < nx;
+  const bool act[2] = {own && ja < ny, own && ja + 1 < ny};
+  const int shift = G::shift(i0);
 
-  R.start(P, maps.m, kbeg, kend, i0, j0, (P.wait_fault & WF_FLOW_RING) != 0);
+  Rg.start(P, maps.m, kbeg, kend, i0, j0, (P.wait_fault & WF_FLOW_RING) != 0);
 
-  // wait for plane kk and overwrite its out-of-domain cells (all cells of a
-  // ghost plane or of a tile overhanging the domain end, else the perimeter
-  // of a tile on the boundary)
-  auto acquire = [&](int kk, bool refill) -> bool {
-    if (!R.wait(kk)) return false;
-    if (refill && tid == 0) R.refill(P, maps.m, kk);
+  // set the ghost cells of plane kk, which has landed: those of a tile on the
+  // boundary, all of a plane beyond a periodic z side; a plane beyond a z wall is
+  // filled from the plane next to it by zwall
+  const bool zper = P.bc[2] == BC_PERIODIC;
+  auto ghosts = [&](int kk) {
     const bool ghost_plane = kk < 0 || kk >= nz;
-    if (!ghost_plane && !edge_tile) return true;
+    if (ghost_plane ? !zper : !edge_tile) return;
     real* pl[NRAW_FLOW];
 #pragma unroll
-    for (int f = 0; f < NRAW_FLOW; ++f) pl[f] = R.plane(kk, f);
-    const bool full = ghost_plane || ragged;
-    const int ncell = full ? SX * SYv : perim<SYv>();
-    for (int q = tid; q < ncell; q += FLOW_NTHR) {
-      int lx, ly;
-      if (full) { ly = q / SX; lx = q - ly * SX; }
-      else perim_cell<SYv>(q, lx, ly);
-      const int gi = i0 - 1 + lx, gj = j0 - 1 + ly;
-      if (ghost_plane || gi < 0 || gi >= nx || gj < 0 || gj >= ny) {
+    for (int f = 0; f < NRAW_FLOW; ++f) pl[f] = Rg.plane(kk, f) + shift;
+    if (ghost_plane) {
+      for (int q = tid; q < 32 * SYv; q += FLOW_NTHR) {
+        const int ly = q >> 5, lx = q & 31;
         const int e = G::at(lx, ly);
-        const int ci = clampi(gi, -1, nx), cj = clampi(gj, -1, ny);
+        const int ci = clampi(i0 - 1 + lx, -1, nx), cj = clampi(j0 - 1 + ly, -1, ny);
         pl[R_P][e] = ld_cen(A.q[0], P, ci, cj, kk);
         pl[R_U][e] = ld_face<0>(A.q[1], P, ci, cj, kk);
         pl[R_V][e] = ld_face<1>(A.q[2], P, ci, cj, kk);
@@ -258,82 +155,233 @@ __global__ void __launch_bounds__(FLOW_NTHR, FLOW_MINB) flow3d_kernel(const __gr
         pl[R_PHI][e] = ld_cen(A.phi, P, ci, cj, kk);
         pl[R_MU][e] = ld_cen(A.mu, P, ci, cj, kk);
       }
+    } else {
+      static_assert(ghost_count<SYv, 32>() <= FLOW_NTHR, "a ghost cell per thread");
+      int lx, ly;
+      if (tid < ghost_count<SYv, 32>() && ghost_cell<SYv, 32>(P, i0, j0, tid, lx, ly)) {
+        const int e = G::at(lx, ly), gi = i0 - 1 + lx, gj = j0 - 1 + ly;
+        pl[R_P][e] = ghost_value<G>(K_CEN, pl[R_P], A.q[0], P, i0, j0, gi, gj, kk);
+        pl[R_U][e] = ghost_value<G>(K_FACE0, pl[R_U], A.q[1], P, i0, j0, gi, gj, kk);
+        pl[R_V][e] = ghost_value<G>(K_FACE1, pl[R_V], A.q[2], P, i0, j0, gi, gj, kk);
+        pl[R_W][e] = ghost_value<G>(K_FACE2, pl[R_W], A.q[3], P, i0, j0, gi, gj, kk);
+        pl[R_PHI][e] = ghost_value<G>(K_CEN, pl[R_PHI], A.phi, P, i0, j0, gi, gj, kk);
+        pl[R_MU][e] = ghost_value<G>(K_CEN, pl[R_MU], A.mu, P, i0, j0, gi, gj, kk);
+      }
     }
     fence_proxy_async_smem();
-    return true;
+  };
+  // the plane kk beyond a z wall from the plane next to it, after a barrier that
+  // follows that plane's ghost writes
+  auto zwall = [&](int kk) {
+    const int from = kk < 0 ? 0 : nz - 1;
+    for (int q = tid; q < G::BX * SYv; q += FLOW_NTHR) {
+      Rg.plane(kk, R_P)[q] = Rg.plane(from, R_P)[q];
+      Rg.plane(kk, R_U)[q] = zwall_value<K_FACE0>(P, Rg.plane(from, R_U)[q]);
+      Rg.plane(kk, R_V)[q] = zwall_value<K_FACE1>(P, Rg.plane(from, R_V)[q]);
+      Rg.plane(kk, R_W)[q] = real(0);
+      Rg.plane(kk, R_PHI)[q] = Rg.plane(from, R_PHI)[q];
+      Rg.plane(kk, R_MU)[q] = Rg.plane(from, R_MU)[q];
+    }
+    fence_proxy_async_smem();
   };
 
-  if (!acquire(kbeg - 1, false)) { R.fail(err, kbeg - 1); return; }
-  if (!acquire(kbeg, false)) { R.fail(err, kbeg); return; }
-  const real* smr = reinterpret_cast<const real*>(smraw);
-  const int raw0 = (int)(R.raw - smr);
-  const int cell0 = G::at(tx + 1, 2 * ty + 1);
-  using Ops = FlowOpsZ<real, RingTile<real, PAVG>>;
-  // the +z side terms of the cells of plane kbeg - 1 (planes kbeg - 1 and kbeg
-  // only), after every thread's writes of the two planes' out-of-domain cells
+  if (!Rg.wait(kbeg - 1)) { Rg.fail(err, kbeg - 1); return; }
+  ghosts(kbeg - 1);
+  if (!Rg.wait(kbeg)) { Rg.fail(err, kbeg); return; }
+  ghosts(kbeg);
+  // after every thread's writes of the two planes' ghost cells
   if (edge_tile || kbeg == 0 || kbeg + 1 >= nz) __syncthreads();
-  ZCarry<real> zc[2];
-#pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    RingTile<real, PAVG> S;
-    S.sm = smr;
-    S.P = &P;
-#pragma unroll
-    for (int dz = -1; dz <= 1; ++dz) S.r[dz + 1] = raw0 + R.slot(kbeg - 1 + dz) * NRAW_FLOW * G::PE + cell0 + r * G::BX;
-    Ops::plus_z(S, P, Ops::divsum(S, P, 0, 0, 0), zc[r]);
+  if (kbeg == 0 && !zper) {
+    zwall(-1);
+    __syncthreads();
   }
+
+  const real* smr = reinterpret_cast<const real*>(smraw);
+  const int cell0 = (int)(Rg.raw - smr) + shift + G::at(tx, 2 * ty + 1);
+  auto base = [&](int kk) { return cell0 + Rg.slot(kk) * NRAW_FLOW * G::PE; };
+  // staged field f at row r, column offset dx of the plane at base b
+  auto S = [&](int b, int f, int r, int dx) { return smr[b + f * G::PE + r * G::BX + dx]; };
+  auto left = [&](real v) { return __shfl_up_sync(FULL, v, 1); };
+  auto right = [&](real v) { return __shfl_down_sync(FULL, v, 1); };
+  const real emd = P.eta_d * P.inv_dx2, emm = P.eta_m * P.inv_dx2;
+  const real bulk = P.bulk ? real(1) : real(0);
+
+  auto material = [&](int b, FlowMat<real, R>& m) {
+#pragma unroll
+    for (int r = -1; r <= R; ++r) {
+      const real ph = S(b, R_PHI, r, 0);
+      m.eta[r + 1] = fma(emd, ph, emm);
+      const real rho = rho_of(P, ph);
+      if (r < R) m.rho[r + 1] = rho;
+      m.nu[r + 1] = quot_rho(m.eta[r + 1], rho);
+      m.sx[r + 1] = m.eta[r + 1] + left(m.eta[r + 1]);
+      if (r >= 0) m.sy[r] = m.eta[r + 1] + m.eta[r];
+    }
+  };
+  // dx div u of the cell in row r of the plane at b, n above it
+  auto divsum = [&](int b, int n, int r) {
+    return ((S(b, R_U, r, 1) - S(b, R_U, r, 0)) + (S(b, R_V, r + 1, 0) - S(b, R_V, r, 0))) +
+           (S(n, R_W, r, 0) - S(b, R_W, r, 0));
+  };
+  // bD: the bulk viscosity's share of the divergence, rows -1 .. R-1
+  auto above = [&](int b, int n, const FlowMat<real, R>& mc, const FlowMat<real, R>& mn, const real* bD,
+                   FlowZ<real, R>& z) {
+#pragma unroll
+    for (int r = 0; r <= R; ++r)
+      z.tyz[r] = (mc.sy[r] + mn.sy[r]) *
+                 ((S(n, R_V, r, 0) - S(b, R_V, r, 0)) + (S(n, R_W, r, 0) - S(n, R_W, r - 1, 0)));
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      z.txz[r] = (mc.sx[r + 1] + mn.sx[r + 1]) *
+                 ((S(n, R_U, r, 0) - S(b, R_U, r, 0)) + (S(n, R_W, r, 0) - S(n, R_W, r, -1)));
+      const real dw = S(n, R_W, r, 0) - S(b, R_W, r, 0);
+      z.tz[r] = mc.eta[r + 1] * fma(real(2), dw, bD[r + 1]);
+      z.rho[r] = mc.rho[r + 1];
+      z.fz[r] = (mc.nu[r + 1] + mn.nu[r + 1]) * (S(n, R_P, r, 0) - S(b, R_P, r, 0));
+      if (PAVG) {
+        const real yp = fma(real(4), S(b, R_P, r, 0), S(b, R_P, r + 1, 0) + S(b, R_P, r - 1, 0));
+        z.xy[r] = fma(real(4), yp, left(yp) + right(yp));
+      }
+    }
+  };
+
+  FlowMat<real, R> mc;
+  FlowZ<real, R> zp;
+  {
+    FlowMat<real, R> mm;
+    material(base(kbeg - 1), mm);
+    material(base(kbeg), mc);
+    real bD[R + 1];
+#pragma unroll
+    for (int r = 0; r < R; ++r) bD[r + 1] = bulk * divsum(base(kbeg - 1), base(kbeg), r);
+    above(base(kbeg - 1), base(kbeg), mm, mc, bD, zp);
+  }
+  const real gfac = P.inv_dx * (PAVG ? real(1.0 / 36.0) : real(1));
+  const real c_st = -P.sigma * P.inv_2dx;
+  const real q2 = real(0.25);
   long long id = lin(P, i, ja, kbeg);
   for (int k = kbeg; k < kend; ++k, id += P.sz) {
-    real q0v[2][4];
+    real q0v[R][4];
     if (MODE == 2) {
 #pragma unroll
-      for (int r = 0; r < 2; ++r)
+      for (int r = 0; r < R; ++r)
         if (act[r]) {
 #pragma unroll
           for (int f = 0; f < 4; ++f) q0v[r][f] = A.q0[f][id + r * P.sy];
         }
     }
-    if (!acquire(k + 1, true)) { R.fail(err, k + 1); return; }
-    // the threads' writes of out-of-domain cells must be seen by all before the
-    // stencil reads them; a plane that needed none is visible to every thread
-    // after its own wait on the plane's barrier
+    if (!Rg.wait(k + 1)) { Rg.fail(err, k + 1); return; }
+    Rg.refill(P, maps.m, k + 1);
+    ghosts(k + 1);
+    // the threads' writes of ghost cells must be seen by all before the stencil
+    // reads them; a plane that needed none is visible to every thread after
+    // its own wait on the plane's barrier
+    if (k + 1 == nz && !zper) zwall(nz);  // (plane nz - 1 was set and read in the last turn)
     if (edge_tile || k + 1 >= nz) __syncthreads();
-    real out[2][4];
+    const int bm = base(k - 1), bc = base(k), bn = base(k + 1);
+    FlowMat<real, R> mn;
+    FlowZ<real, R> zc;
+    material(bn, mn);
+    real out[R][4];
+    // terms of rows -1 .. R the two cells share
+    real D[R + 1], bD[R + 1], Ty[R + 1], txy[R + 1], fy[R + 1], zpr[R + 2], xz[R + 1];
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      RingTile<real, PAVG> S;
-      S.sm = smr;
-      S.P = &P;
+    for (int r = -1; r < R; ++r) {
+      D[r + 1] = divsum(bc, bn, r);
+      bD[r + 1] = bulk * D[r + 1];
+      Ty[r + 1] = mc.eta[r + 1] * fma(real(2), S(bc, R_V, r + 1, 0) - S(bc, R_V, r, 0), bD[r + 1]);
+    }
+    above(bc, bn, mc, mn, bD, zc);
 #pragma unroll
-      for (int dz = -1; dz <= 1; ++dz) S.r[dz + 1] = raw0 + R.slot(k + dz) * NRAW_FLOW * G::PE + cell0 + r * G::BX;
-      const real D0 = Ops::divsum(S, P, 0, 0, 0);
-      ZCarry<real> zo;
-      Ops::plus_z(S, P, D0, zo);
+    for (int r = 0; r <= R; ++r) {
+      txy[r] = (mc.sx[r + 1] + mc.sx[r]) * ((S(bc, R_U, r, 0) - S(bc, R_U, r - 1, 0)) +
+                                            (S(bc, R_V, r, 0) - S(bc, R_V, r, -1)));
+      fy[r] = (mc.nu[r + 1] + mc.nu[r]) * (S(bc, R_P, r, 0) - S(bc, R_P, r - 1, 0));
+    }
+    if (PAVG) {
+#pragma unroll
+      for (int r = -1; r <= R; ++r) zpr[r + 1] = fma(real(4), S(bc, R_P, r, 0), S(bm, R_P, r, 0) + S(bn, R_P, r, 0));
+#pragma unroll
+      for (int r = -1; r < R; ++r) xz[r + 1] = fma(real(4), zpr[r + 1], left(zpr[r + 1]) + right(zpr[r + 1]));
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const real p0 = S(bc, R_P, r, 0), u0 = S(bc, R_U, r, 0), v0 = S(bc, R_V, r, 0), w0 = S(bc, R_W, r, 0);
+      const real ur = S(bc, R_U, r, 1), ul = S(bc, R_U, r, -1), wn = S(bn, R_W, r, 0);
+      // pressure
+      const real fx = (mc.nu[r + 1] + left(mc.nu[r + 1])) * (p0 - S(bc, R_P, r, -1));
+      const real diff = ((right(fx) - fx) + (fy[r + 1] - fy[r])) + (zc.fz[r] - zp.fz[r]);
+      const real Lp = fma(real(0.5), diff, -(mc.rho[r + 1] * P.cs2 * (D[r + 1] * P.inv_dx)));
+      const real ph0 = S(bc, R_PHI, r, 0), mu0 = S(bc, R_MU, r, 0);
+      // u on the low x face
       real L[4];
-      L[0] = Ops::rate_p(S, P, D0, zc[r], zo);
-      L[1] = Ops::template rate_vel<0>(S, P, D0, zc[r], zo);
-      L[2] = Ops::template rate_vel<1>(S, P, D0, zc[r], zo);
-      L[3] = Ops::template rate_vel<2>(S, P, D0, zc[r], zo);
-      zc[r] = zo;
+      L[0] = Lp;
+      {
+        const real Tx = mc.eta[r + 1] * fma(real(2), ur - u0, bD[r + 1]);
+        real F = fma(q2, (txy[r + 1] - txy[r]) + (zc.txz[r] - zp.txz[r]), Tx - left(Tx));
+        real g;
+        if (PAVG) {
+          const real yz = fma(real(4), zpr[r + 1], zpr[r + 2] + zpr[r]);
+          g = yz - left(yz);
+        } else {
+          g = p0 - S(bc, R_P, r, -1);
+        }
+        F = fma(-g, gfac, F);
+        F = fma(c_st * (ph0 + S(bc, R_PHI, r, -1)), mu0 - S(bc, R_MU, r, -1), F);
+        const real rb = mc.rho[r + 1] + left(mc.rho[r + 1]);
+        F = fma(fma(real(0.5), rb, -P.rho_ref), P.g[0], F);
+        const real V4 = (v0 + S(bc, R_V, r, -1)) + (S(bc, R_V, r + 1, 0) + S(bc, R_V, r + 1, -1));
+        const real W4 = (w0 + S(bc, R_W, r, -1)) + (wn + S(bn, R_W, r, -1));
+        const real tr = fma(V4, S(bc, R_U, r + 1, 0) - S(bc, R_U, r - 1, 0), W4 * (S(bn, R_U, r, 0) - S(bm, R_U, r, 0)));
+        const real conv = fma(u0, ur - ul, q2 * tr);
+        L[1] = fma(-conv, P.inv_2dx, quot_rho(real(2) * F, rb));
+      }
+      // v on the low y face
+      {
+        real F = fma(q2, (right(txy[r]) - txy[r]) + (zc.tyz[r] - zp.tyz[r]), Ty[r + 1] - Ty[r]);
+        const real g = PAVG ? xz[r + 1] - xz[r] : p0 - S(bc, R_P, r - 1, 0);
+        F = fma(-g, gfac, F);
+        F = fma(c_st * (ph0 + S(bc, R_PHI, r - 1, 0)), mu0 - S(bc, R_MU, r - 1, 0), F);
+        const real rb = mc.rho[r + 1] + mc.rho[r];
+        F = fma(fma(real(0.5), rb, -P.rho_ref), P.g[1], F);
+        const real uy = u0 + S(bc, R_U, r - 1, 0);
+        const real U4 = uy + right(uy);
+        const real W4 = (w0 + S(bc, R_W, r - 1, 0)) + (wn + S(bn, R_W, r - 1, 0));
+        const real tr = fma(U4, S(bc, R_V, r, 1) - S(bc, R_V, r, -1), W4 * (S(bn, R_V, r, 0) - S(bm, R_V, r, 0)));
+        const real conv = fma(v0, S(bc, R_V, r + 1, 0) - S(bc, R_V, r - 1, 0), q2 * tr);
+        L[2] = fma(-conv, P.inv_2dx, quot_rho(real(2) * F, rb));
+      }
+      // w on the low z face
+      {
+        real F = fma(q2, (right(zp.txz[r]) - zp.txz[r]) + (zp.tyz[r + 1] - zp.tyz[r]), zc.tz[r] - zp.tz[r]);
+        const real g = PAVG ? zc.xy[r] - zp.xy[r] : p0 - S(bm, R_P, r, 0);
+        F = fma(-g, gfac, F);
+        F = fma(c_st * (ph0 + S(bm, R_PHI, r, 0)), mu0 - S(bm, R_MU, r, 0), F);
+        const real rb = mc.rho[r + 1] + zp.rho[r];
+        F = fma(fma(real(0.5), rb, -P.rho_ref), P.g[2], F);
+        const real uz = u0 + S(bm, R_U, r, 0);
+        const real U4 = uz + right(uz);
+        const real V4 = (v0 + S(bm, R_V, r, 0)) + (S(bc, R_V, r + 1, 0) + S(bm, R_V, r + 1, 0));
+        const real tr = fma(U4, S(bc, R_W, r, 1) - S(bc, R_W, r, -1),
+                            V4 * (S(bc, R_W, r + 1, 0) - S(bc, R_W, r - 1, 0)));
+        const real conv = fma(w0, wn - S(bm, R_W, r, 0), q2 * tr);
+        L[3] = fma(-conv, P.inv_2dx, quot_rho(real(2) * F, rb));
+      }
       // faces on a wall are never updated
       if (P.bc[0] != BC_PERIODIC && i == 0) L[1] = real(0);
       if (P.bc[1] != BC_PERIODIC && ja + r == 0) L[2] = real(0);
       if (P.bc[2] != BC_PERIODIC && k == 0) L[3] = real(0);
-      const int F[4] = {F_P, F_U, F_V, F_W};
+      const real q[4] = {p0, u0, v0, w0};
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
-        if (MODE == 0) {
-          out[r][f] = L[f];
-        } else {
-          const real q = S(F[f], 0, 0, 0);
-          if (MODE == 1) out[r][f] = q + P.dt * L[f];
-          else out[r][f] = A.a * q0v[r][f] + A.b * (q + P.dt * L[f]);
-        }
+        if (MODE == 0) out[r][f] = L[f];
+        else if (MODE == 1) out[r][f] = fma(P.dt, L[f], q[f]);
+        else out[r][f] = fma(A.a, q0v[r][f], A.b * fma(P.dt, L[f], q[f]));
       }
     }
     // stores after both cells, so that nothing separates their shared loads
 #pragma unroll
-    for (int r = 0; r < 2; ++r)
+    for (int r = 0; r < R; ++r)
       if (act[r]) {
 #pragma unroll
         for (int f = 0; f < 4; ++f) A.out[f][id + r * P.sy] = out[r][f];
@@ -342,12 +390,14 @@ __global__ void __launch_bounds__(FLOW_NTHR, FLOW_MINB) flow3d_kernel(const __gr
     // CH step forms the time-centred cell velocity with half the loads
     if (MODE == 2 && A.usum[0]) {
 #pragma unroll
-      for (int r = 0; r < 2; ++r)
+      for (int r = 0; r < R; ++r)
         if (act[r]) {
 #pragma unroll
           for (int a = 0; a < 3; ++a) A.usum[a][id + r * P.sy] = q0v[r][1 + a] + out[r][1 + a];
         }
     }
+    mc = mn;
+    zp = zc;
   }
 }
 
@@ -365,8 +415,9 @@ cudaError_t launch_flow_stage(const KParams<real>& P, const FlowArgs<real>& A, i
   cudaError_t e;
   if constexpr (DIM == 3) {
     constexpr int RING = flow_ring<real>();
-    const size_t sm = ring_smem_bytes<real, NRAW_FLOW, 0, RING, FLOW_K3_SY>();
+    const size_t sm = 256 + sizeof(real) * (size_t)FlowGeom<real, FLOW_K3_SY>::PE * RING * NRAW_FLOW;
     blk.y = FLOW_TY;
+    grd.x = (P.n[0] + FLOW_K3_TX - 1) / FLOW_K3_TX;
     grd.y = (P.n[1] + FLOW_K3_TY - 1) / FLOW_K3_TY;
 #define GPE2P_FLOW3_CASE(M)                                                                                 \
   if (P.pavg) {                                                                                             \

@@ -26,6 +26,8 @@ constexpr int FLOW_NTHR = TX * FLOW_TY;
 constexpr int FLOW_K3_TY = 2 * FLOW_TY;
 constexpr int FLOW_K3_SY = FLOW_K3_TY + 2;
 constexpr int FLOW_MINB = 16 / FLOW_TY;
+constexpr int FLOW_MINB64 = 2;    // FP64: 255 registers a thread, no spills
+constexpr int FLOW_K3_TX = 30;    // columns of a block: the 32 lanes but one on each side
 
 // the blocks of the 3D CH stage and of mu, likewise (2 CH_TY and MU_CPT MU_TY
 // rows of cells), and the blocks of each that fit on an SM: the FP32 CH stage

@@ -44,6 +44,21 @@ struct RingGeom {
   // element (lx, ly) of the staged region (lx, ly in [0, SX) x [0, SYv)): global
   // cell (i0 - 1 + lx, j0 - 1 + ly)
   __device__ __forceinline__ static int at(int lx, int ly) { return ly * BX + lx + A - 1; }
+  __device__ __forceinline__ static int start(int i0) { return i0 - A; }
+};
+
+// The flow stage's staged region: 32 columns, the block's 30 and one on each side,
+// one per lane.  The box starts on the 16-byte boundary at or below the first;
+// element (lx, ly) lies at at(lx, ly) + shift(i0).
+template <typename real, int SYv>
+struct FlowGeom {
+  static constexpr int A = 16 / (int)sizeof(real);
+  static constexpr int BX = 32 + A;
+  static constexpr int PE = ((BX * SYv * (int)sizeof(real) + 127) / 128) * 128 / (int)sizeof(real);
+  static constexpr uint32_t BOX_BYTES = BX * SYv * sizeof(real);
+  __device__ __forceinline__ static int at(int lx, int ly) { return ly * BX + lx; }
+  __device__ __forceinline__ static int start(int i0) { return (i0 - 1) & ~(A - 1); }
+  __device__ __forceinline__ static int shift(int i0) { return (i0 - 1) & (A - 1); }
 };
 
 template <int NMAP>
@@ -51,35 +66,42 @@ struct Maps {
   CUtensorMap m[NMAP];
 };
 
-// The pipeline state of one block.  NRAW fields are staged per plane; RING is
-// a power of two so that slots and phases are masks and shifts.
-template <typename real, int NRAW, int RING, int SYv = SY>
+// The pipeline state of one block.  NRAW fields are staged per plane; lane 0 of
+// each of the first NISS warps issues its share of a plane's copies.  (A single
+// issuing thread spends about a hundred instructions a plane on six copies,
+// which the block's other warps wait out at the next barrier: shared, a step of
+// 256 x 256 x 512 takes 1.2 % less.)
+template <typename real, int NRAW, int RING, int SYv = SY, typename Geom = RingGeom<real, SYv>, int NISS = 1>
 struct Ring {
-  static_assert((RING & (RING - 1)) == 0 && RING >= 4, "RING must be a power of two >= 4");
-  static constexpr int LOG2 = RING == 4 ? 2 : (RING == 8 ? 3 : 4);
-  using G = RingGeom<real, SYv>;
+  static_assert(RING >= 4 && RING <= 8, "slots of a ring (its barriers take 64 bytes)");
+  using G = Geom;
   uint64_t* bar;  // RING barriers
   real* raw;      // RING x NRAW x PE
   int first, last;  // planes kbeg-1 .. kend (inclusive)
   int i0, j0;
+  int x0;           // first staged column (16-byte aligned)
   int issued;       // last plane issued
   bool lose_first;  // test switch: report the wait for the first plane as timed out
-  __device__ __forceinline__ int slot(int kk) const { return (int)((unsigned)(kk - first) & (RING - 1)); }
-  __device__ __forceinline__ uint32_t parity(int kk) const { return ((unsigned)(kk - first) >> LOG2) & 1u; }
+  __device__ __forceinline__ int slot(int kk) const { return (int)((unsigned)(kk - first) % RING); }
+  __device__ __forceinline__ uint32_t parity(int kk) const { return ((unsigned)(kk - first) / RING) & 1u; }
   __device__ __forceinline__ real* plane(int kk, int f) const { return raw + ((size_t)slot(kk) * NRAW + f) * G::PE; }
 
-  // thread 0: start the copies of plane kk (or, for a ghost plane, just arrive)
+  // an issuing thread: start its copies of plane kk (or, for a ghost plane, just arrive)
   __device__ __forceinline__ void issue(const KParams<real>& P, const CUtensorMap* maps, int kk) {
     uint64_t* b = &bar[slot(kk)];
-    if (kk >= 0 && kk < P.n[2]) {
-      mbar_arrive_expect_tx(b, NRAW * G::BOX_BYTES);
+    const int me = threadIdx.y;
+    if (kk >= 0 && kk < P.n[2] && (NISS == 1 || me < NRAW)) {
+      const int mine = NISS == 1 ? NRAW : (NRAW - 1 - me) / NISS + 1;
+      mbar_arrive_expect_tx(b, mine * G::BOX_BYTES);
 #pragma unroll
-      for (int f = 0; f < NRAW; ++f) tma_load_3d(plane(kk, f), &maps[f], i0 - G::A, j0 - 1, kk, b);
+      for (int f = 0; f < NRAW; f += NISS)
+        if (NISS == 1 || f + me < NRAW) tma_load_3d(plane(kk, f + me), &maps[f + me], x0, j0 - 1, kk, b);
     } else {
       mbar_arrive(b);
     }
     issued = kk;
   }
+  __device__ __forceinline__ bool issuer() const { return threadIdx.x == 0 && threadIdx.y < NISS; }
 
   // lose: the test switch of the timeout path (the wait for the first plane
   // still completes, so no copy is left in flight, and then reports a timeout)
@@ -90,13 +112,14 @@ struct Ring {
     last = kend;
     i0 = i0_;
     j0 = j0_;
+    x0 = G::start(i0_);
     issued = first - 1;
     if (threadIdx.x == 0 && threadIdx.y == 0) {
-      for (int s = 0; s < RING; ++s) mbar_init(&bar[s], 1);
+      for (int s = 0; s < RING; ++s) mbar_init(&bar[s], NISS);
       fence_mbar_init();
     }
     __syncthreads();
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
+    if (issuer()) {
       const int upto = min(last, first + RING - 1);
       for (int kk = first; kk <= upto; ++kk) issue(P, maps, kk);
     }
@@ -109,11 +132,11 @@ struct Ring {
     return !__syncthreads_or(!ok);
   }
 
-  // thread 0, after the wait for plane kk (every thread is then done with
+  // all threads, after the wait for plane kk (every thread is then done with
   // plane kk - 3): start plane kk - 3 + RING in the freed slot
   __device__ __forceinline__ void refill(const KParams<real>& P, const CUtensorMap* maps, int kk) {
     const int nk = kk - 3 + RING;
-    if (nk <= last && nk > issued) issue(P, maps, nk);
+    if (issuer() && nk <= last && nk > issued) issue(P, maps, nk);
   }
 
   // after a timeout: record it, let this block's copies in flight land, return
@@ -125,17 +148,71 @@ struct Ring {
   }
 };
 
-// the staged cells of a plane that can lie outside the domain: all of them on
-// a ghost plane, else the one-cell perimeter of the staged region (SYv rows)
-template <int SYv = SY>
-constexpr int perim() { return 2 * SX + 2 * (SYv - 2); }
-constexpr int PERIM = perim<SY>();
-template <int SYv = SY>
-__device__ __forceinline__ void perim_cell(int q, int& lx, int& ly) {
-  if (q < SX) { lx = q; ly = 0; }
-  else if (q < 2 * SX) { lx = q - SX; ly = SYv - 1; }
-  else if (q < 2 * SX + SYv - 2) { lx = 0; ly = q - 2 * SX + 1; }
-  else { lx = SX - 1; ly = q - 2 * SX - (SYv - 2) + 1; }
+// The ghost cells of a staged plane inside the domain: the columns at -1 and nx and
+// the rows at -1 and ny of a tile that reaches them (staged cells further out are
+// read by no cell of the domain).  Candidate q < ghost_count<SYv>() of the tile
+// at (i0, j0): its staged position, or false if the tile does not have it.
+template <int SYv, int SXv = SX>
+constexpr int ghost_count() { return 2 * SYv + 2 * SXv; }
+template <int SYv, int SXv = SX, typename real>
+__device__ __forceinline__ bool ghost_cell(const KParams<real>& P, int i0, int j0, int q, int& lx, int& ly) {
+  if (q < 2 * SYv) {
+    ly = q >> 1;
+    lx = (q & 1) ? P.n[0] - i0 + 1 : 0;
+    return ((q & 1) ? lx < SXv : i0 == 0) && j0 - 1 + ly <= P.n[1];
+  }
+  q -= 2 * SYv;
+  lx = q >> 1;
+  ly = (q & 1) ? P.n[1] - j0 + 1 : 0;
+  return ((q & 1) ? ly < SYv : j0 == 0) && i0 - 1 + lx <= P.n[0];
+}
+
+// The value of a ghost cell (gi, gj) of plane kk.  Across a wall it mirrors a cell
+// that the same plane holds in shared memory (pl: the staged field): a copy there
+// costs a tile at the boundary nothing, while the global loads of ld_kind cost
+// it their latency in every plane.  Across a periodic side the other end
+// of the domain is read.
+template <typename G, typename real>
+__device__ __forceinline__ real ghost_value(int kind, const real* pl, const real* __restrict__ f,
+                                            const KParams<real>& P, int i0, int j0, int gi, int gj, int kk) {
+  // out of the domain across a wall, and across a periodic side
+  const bool ax = gi < 0 || gi >= P.n[0], ay = gj < 0 || gj >= P.n[1];
+  const bool px = ax && P.bc[0] == BC_PERIODIC, py = ay && P.bc[1] == BC_PERIODIC;
+  const bool ox = ax && !px, oy = ay && !py;
+  int x = px ? wrap1(gi, P.n[0]) : clampi(gi, 0, P.n[0] - 1), y = py ? wrap1(gj, P.n[1]) : clampi(gj, 0, P.n[1] - 1);
+  bool neg = false;
+  if (kind == K_FACE0 || kind == K_FACE1) {
+    // odd about a wall face along the component's axis, zero on it
+    const bool along_x = kind == K_FACE0;
+    if (along_x ? ox : oy) {
+      const int g = along_x ? gi : gj, n = P.n[along_x ? 0 : 1];
+      if (g >= n || n < 2) return real(0);
+      if (along_x) x = 1;
+      else y = 1;
+      neg = true;
+    }
+    if ((along_x ? oy : ox) && P.bc[along_x ? 1 : 0] == BC_NOSLIP) neg = !neg;
+  } else if (kind == K_FACE2) {
+    if (ox && P.bc[0] == BC_NOSLIP) neg = !neg;
+    if (oy && P.bc[1] == BC_NOSLIP) neg = !neg;
+  } else if (kind == K_CVEC0) {
+    neg = ox;
+  } else if (kind == K_CVEC1) {
+    neg = oy;
+  }
+  const real v = px || py ? f[lin(P, x, y, kk)] : pl[G::at(x - i0 + 1, y - j0 + 1)];
+  return neg ? -v : v;
+}
+
+// The plane beyond a z wall, field by field: dst from src, the plane next to the
+// wall with its own ghosts in place.  (The w face outside is read by no
+// updated face; on the high wall, w = 0.)
+template <int KIND, typename real>
+__device__ __forceinline__ real zwall_value(const KParams<real>& P, real v) {
+  if (KIND == K_FACE2) return real(0);
+  if (KIND == K_CVEC2) return -v;
+  if (KIND == K_FACE0 || KIND == K_FACE1) return P.bc[2] == BC_NOSLIP ? -v : v;
+  return v;
 }
 
 // shared-memory bytes of a kernel with NRAW staged and NDER derived fields

@@ -438,25 +438,6 @@ __device__ __forceinline__ void ch_ghosts(const KParams<real>& P, real* f, int g
   }
 }
 
-// phi + lo + (d1 + d2) / 2 as a high/low pair, in FP32 pairs: the two sums that
-// carry rounding (d1 + d2, phi + half of it) are taken with their errors
-// (two-sum, Knuth), so what is lost is the rounding of the low parts, about
-// 2^-48 of phi, the precision the pair itself has.  GB300's FP64 pipe is 64
-// times narrower than its FP32 one.
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float t = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
-}
-__device__ __forceinline__ void pair_update(float ph, float lo, float d1, float d2, float& hi, float& low) {
-  float s, se, t, te;
-  two_sum(d1, d2, s, se);
-  two_sum(ph, 0.5f * s, t, te);
-  const float c = __fadd_rn(te, __fadd_rn(lo, 0.5f * se));
-  hi = __fadd_rn(t, c);
-  low = __fadd_rn(__fsub_rn(t, hi), c);
-}
-
 // The whole TVD-RK2 CH step of the advective form on the tile of FUSED_X x
 // ch_rows(NW R) cells at (i0, j0): phi_1, mu(phi_1), phi^{n+3/2} and its mu,
 // each on one cell less on every side.  sm: ch_fused_smem reals.
@@ -629,7 +610,7 @@ __device__ __forceinline__ void ch2d_fused_tile(const KParams<real>& P, const CH
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       if (A.lo) {
-        pair_update(pn[r], lo[r], d1[r], mul_rn(P.dt, L[r]), hi[r], low[r]);
+        pair_half(pn[r], lo[r], d1[r], mul_rn(P.dt, L[r]), hi[r], low[r]);
       } else {
         hi[r] = fma(real(0.5), pn[r], mul_rn(real(0.5), fma(P.dt, L[r], f1[r])));
         low[r] = real(0);
