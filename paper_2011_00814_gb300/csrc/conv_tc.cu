@@ -130,20 +130,48 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t v[8]) {
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-__device__ __forceinline__ float silu_f(float z) { return __fdividef(z, 1.0f + __expf(-z)); }
+// z / (1 + exp(-z)); the denominator is at least 1, so the reciprocal needs none
+// of the general quotient's range handling (an infinite one gives zero)
+__device__ __forceinline__ float silu_f(float z) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + __expf(-z)));
+  return z * r;
+}
 
 struct TileGeom {
   int b, y0, x0;
 };
 
-__device__ __forceinline__ TileGeom tile_of(int t, int tiles_x, int tiles_y) {
-  TileGeom g;
-  const int tx = t % tiles_x;
-  t /= tiles_x;
-  g.y0 = (t % tiles_y) * TH;
-  g.b = t / tiles_y;
-  g.x0 = tx * TW;
-  return g;
+// A CTA's tiles t, t + gridDim.x, ... in (x, y, image) coordinates, stepped by
+// additions: divisions by the tile counts and the image size for every tile
+// and window entry kept a producer warp busy for most of a tile of a 32-channel
+// layer (32 -> 32 channels, 256 x 256, batch 8, ncu: 41.7 us with divisions, 32.1
+// without, with the biases in shared memory).
+struct TileIter {
+  int tx, ty, b, sx, sy, sb, nx, ny;
+  __device__ __forceinline__ TileIter(int t, int step, int tiles_x, int tiles_y) : nx(tiles_x), ny(tiles_y) {
+    tx = t % nx;
+    ty = (t / nx) % ny;
+    b = t / (nx * ny);
+    sx = step % nx;
+    sy = (step / nx) % ny;
+    sb = step / (nx * ny);
+  }
+  __device__ __forceinline__ TileGeom geom() const { return {b, ty * TH, tx * TW}; }
+  __device__ __forceinline__ void next() {
+    tx += sx;
+    ty += sy;
+    b += sb;
+    if (tx >= nx) { tx -= nx; ++ty; }
+    if (ty >= ny) { ty -= ny; ++b; }
+  }
+};
+
+// v in [-1, n + 17) wrapped into [0, n): one conditional add on an image at
+// least as large as a window (near), else the remainder
+__device__ __forceinline__ int wrap_window(int v, int n, bool near) {
+  if (near) return v < 0 ? v + n : (v >= n ? v - n : v);
+  return wrapm(v, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -189,7 +217,7 @@ __device__ __forceinline__ void cp_async_arrive_noinc(uint64_t* bar) {
 // per epilogue thread (lane m of the tile)
 template <int MODE, int BN>
 __device__ __forceinline__ void epilogue_tile(const ConvArgs& a, uint32_t acc, const TileGeom& tg, int n0, int m,
-                                            int warp) {
+                                            int warp, const float* sbias) {
   const int y = tg.y0 + m / TW, x = tg.x0 + m % TW;
   const bool valid = y < a.H && x < a.W;
   const size_t p = ((size_t)tg.b * a.H + (valid ? y : 0)) * a.W + (valid ? x : 0);
@@ -209,7 +237,7 @@ __device__ __forceinline__ void epilogue_tile(const ConvArgs& a, uint32_t acc, c
       for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[8 * hh + e]);
       if (MODE == 0) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) f[e] += a.bias[n + e];  // the bias sits at any offset of the parameters
+        for (int e = 0; e < 8; ++e) f[e] += sbias[j + 8 * hh + e];
         if (a.z) {
           uint4 zz;
           __nv_bfloat162* zp = reinterpret_cast<__nv_bfloat162*>(&zz);
@@ -259,8 +287,9 @@ __global__ void __launch_bounds__(NTHR) conv3_tc_kernel(const ConvArgs a, int ti
   uint64_t* accf = empty + SMAX;                     // 2: an accumulator's tile is complete (tcgen05.commit)
   uint64_t* acce = accf + 2;                          // 2: an accumulator has been read (the epilogue arrives)
   uint64_t* wbar = acce + 2;                          // the resident weights have landed
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + 512);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + 520);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + 256);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + 264);
+  float* sbias = reinterpret_cast<float*>(sm + 512);  // the block's biases (forward): 4 BN <= 512 bytes
   unsigned char* stages = sm + HEAD;
   const int stage_bytes = A_BYTES + (resident ? 0 : C::BCHUNK);
   unsigned char* wres = stages + ns * stage_bytes;
@@ -300,10 +329,13 @@ __global__ void __launch_bounds__(NTHR) conv3_tc_kernel(const ConvArgs a, int ti
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // (parameters, which no kernel ahead of this one in a dependent launch writes)
+  if (MODE == 0 && tid < BN) sbias[tid] = a.bias[n0 + tid];
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
+  TileIter ti(blockIdx.x, gridDim.x, tiles_x, tiles_y);
 
   if (warp >= EPI_WARPS && warp < MMA_WARP) {
     // ---- producers ----
@@ -335,6 +367,7 @@ __global__ void __launch_bounds__(NTHR) conv3_tc_kernel(const ConvArgs a, int ti
     asm volatile("griddepcontrol.wait;" ::: "memory");
     int s = 0, k = 0, item = 0;
     uint32_t epar = 1;  // parity of the empty phase a stage's next use waits for (none in the first round)
+    const bool near_y = H >= WH - 1, near_x = W >= WH - 1;
     for (int g = 0; g < G; ++g) {
       // the warp leaves together (its lanes meet at __syncwarp below)
       bool stop = *abort_flag != 0;
@@ -344,12 +377,13 @@ __global__ void __launch_bounds__(NTHR) conv3_tc_kernel(const ConvArgs a, int ti
         break;
       }
       if (k == 0) {
-        const TileGeom tg = tile_of(blockIdx.x + item * gridDim.x, tiles_x, tiles_y);
+        const TileGeom tg = ti.geom();
+        ti.next();
 #pragma unroll
         for (int j = 0; j < NWIN; ++j) {
           const int r = r0 + 32 * j;
           const int wy = r / WW, wx = r - wy * WW;
-          int yy = wrapm(tg.y0 + wy - 1, H), xx = wrapm(tg.x0 + wx - 1, W);
+          int yy = wrap_window(tg.y0 + wy - 1, H, near_y), xx = wrap_window(tg.x0 + wx - 1, W, near_x);
           if (a.up) { yy >>= 1; xx >>= 1; }
           wp[j] = src + ((size_t)(tg.b * Hs + yy) * Ws + xx) * lds + soff + 8 * hq;
         }
@@ -434,8 +468,9 @@ __global__ void __launch_bounds__(NTHR) conv3_tc_kernel(const ConvArgs a, int ti
         break;
       }
       tc_fence_after();
-      const TileGeom tg = tile_of(blockIdx.x + item * gridDim.x, tiles_x, tiles_y);
-      epilogue_tile<MODE, BN>(a, tmem + (uint32_t)(buf * BN), tg, n0, warp * 32 + lane, warp);
+      const TileGeom tg = ti.geom();
+      ti.next();
+      epilogue_tile<MODE, BN>(a, tmem + (uint32_t)(buf * BN), tg, n0, warp * 32 + lane, warp, sbias);
       tc_fence_before();
       mbar_arrive(&acce[buf]);
     }
@@ -641,6 +676,8 @@ __global__ void __launch_bounds__(WG_NTHR) wgrad3_tc_kernel(const ConvArgs a, in
     const int xg = tid % C::CG, xr = tid / C::CG, zg = tid % C::OG, zr = tid / C::OG;
     const __nv_bfloat16* xsrc = a.x + a.xoff + ci0 + 8 * xg;
     const __nv_bfloat16* zsrc = a.dz + co0 + 8 * zg;
+    const bool near_y = H >= WH - 1, near_x = W >= WH - 1;
+    TileIter ti(blockIdx.x, gridDim.x, tiles_x, tiles_y);
     int s = 0;
     uint32_t epar = 1;
     for (int it = 0; it < nitems; ++it) {
@@ -650,7 +687,8 @@ __global__ void __launch_bounds__(WG_NTHR) wgrad3_tc_kernel(const ConvArgs a, in
         *abort_flag = 1;
         break;
       }
-      const TileGeom tg = tile_of(blockIdx.x + it * gridDim.x, tiles_x, tiles_y);
+      const TileGeom tg = ti.geom();
+      ti.next();
       unsigned char* X = stages + s * C::STAGE;
       unsigned char* Z = X + C::X_BYTES;
 #pragma unroll 4
@@ -658,7 +696,7 @@ __global__ void __launch_bounds__(WG_NTHR) wgrad3_tc_kernel(const ConvArgs a, in
         const int r = xr + XP * j;
         if (r < WH * WW) {
           const int wy = r / WW, wx = r - wy * WW;
-          int yy = wrapm(tg.y0 + wy - 1, H), xx = wrapm(tg.x0 + wx - 1, W);
+          int yy = wrap_window(tg.y0 + wy - 1, H, near_y), xx = wrap_window(tg.x0 + wx - 1, W, near_x);
           if (a.up) { yy >>= 1; xx >>= 1; }
           cp_async16(X + ((wy * C::CG + xg) * WW + wx) * 16, xsrc + ((size_t)(tg.b * Hs + yy) * Ws + xx) * a.ldx);
         }
