@@ -113,11 +113,15 @@ static int add_conv(gpe2p_net* n, int cin, int cout, int taps, int level) {
 }
 
 static cudaError_t refresh_bf16(gpe2p_net* n) {
+  WeightLayers ls{};
+  static_assert(2 * 6 + 3 * 5 <= 32, "every convolution of the deepest net has its entry");
+  long long rows = 0;
   for (auto& c : n->conv) {
-    cudaError_t e = weights_bf16(n->P + c.w, c.wt, c.wd, c.wtp, c.wdp, c.cout, c.cin, c.taps, n->stream);
-    if (e != cudaSuccess) return e;
+    ls.l[ls.n++] = {n->P + c.w, c.wt, c.wd, c.wtp, c.wdp, c.cout, c.cin, c.taps, rows};
+    rows += (long long)c.cout * c.taps * c.cin / 8;
   }
-  return cudaSuccess;
+  ls.rows = 2 * rows;
+  return weights_bf16(ls, n->stream);
 }
 
 static ConvArgs conv_args(const gpe2p_net* n, const ConvL& c, int B) {
@@ -241,8 +245,7 @@ static cudaError_t backward(gpe2p_net* n, int B) {
     if ((e = bwd(n, n->conv[n->dec_a[l]], B, n->cat[l].v, 2 * c, 0, n->da[l].g, c, 0, n->cat[l].g, 2 * c, 0, 0)) !=
         cudaSuccess)
       return e;
-    if ((e = copy_ch(n->cat[l].g, 2 * c, c, n->eb[l].g, c, 0, npix_at(n, l, B), c, 0, n->stream)) != cudaSuccess)
-      return e;
+    // (the encoder output's gradient stays where it is, the second half of cat[l].g)
     const __nv_bfloat16* dlow = l + 1 <= L - 2 ? n->db[l + 1].v : n->eb[L - 1].v;
     if ((e = bwd(n, n->conv[n->up[l]], B, dlow, cu, 0, n->cat[l].g, 2 * c, 0, n->upx[l].g, cu, 0, 0, 1)) !=
         cudaSuccess)
@@ -253,7 +256,9 @@ static cudaError_t backward(gpe2p_net* n, int B) {
   // encoder, from the bottleneck down
   for (int l = L - 1; l >= 0; --l) {
     const int c = n->ch[l];
-    if ((e = bwd(n, n->conv[n->enc_b[l]], B, n->ea[l].v, c, 0, n->eb[l].g, c, 0, n->ea[l].g, c, 0, 0)) != cudaSuccess)
+    const bool cat = l < L - 1;
+    if ((e = bwd(n, n->conv[n->enc_b[l]], B, n->ea[l].v, c, 0, cat ? n->cat[l].g : n->eb[l].g, cat ? 2 * c : c,
+                 cat ? c : 0, n->ea[l].g, c, 0, 0)) != cudaSuccess)
       return e;
     const __nv_bfloat16* in = l > 0 ? n->pooled[l - 1].v : n->in16.v;
     const int ldin = l > 0 ? n->ch[l - 1] : 16;
@@ -262,7 +267,7 @@ static cudaError_t backward(gpe2p_net* n, int B) {
       return e;
     if (l > 0) {
       const int cp = n->ch[l - 1];
-      if ((e = pool_bwd(n->pooled[l - 1].g, n->eb[l - 1].g, cp, 0, B, n->H >> (l - 1), n->W >> (l - 1), cp, 1,
+      if ((e = pool_bwd(n->pooled[l - 1].g, n->cat[l - 1].g, 2 * cp, cp, B, n->H >> (l - 1), n->W >> (l - 1), cp, 1,
                         n->stream)) != cudaSuccess)
         return e;
     }

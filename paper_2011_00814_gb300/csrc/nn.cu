@@ -258,30 +258,60 @@ __device__ __forceinline__ uint4 ld8(const __nv_bfloat16* p) { return *reinterpr
 __device__ __forceinline__ void st8(__nv_bfloat16* p, const uint4& v) { *reinterpret_cast<uint4*>(p) = v; }
 
 // dZ = dY * silu'(z) (dY read with row stride ldy and channel offset yoff) and
-// db[c] += sum over pixels of the stored dZ; a thread takes 8 channels of a pixel
-__global__ void dsilu_bias_kernel(const __nv_bfloat16* dy, int ldy, int yoff, const __nv_bfloat16* z,
-                                  __nv_bfloat16* dz, long long npix, int c, float* db) {
+// db[c] += sum over pixels of the stored dZ; a thread takes 8 channels of a
+// pixel, PX pixels at a time so that their loads are in flight together.
+// Bound by HBM (three BF16 tensors) and, with the exact exp and reciprocal,
+// nearly as much by issue.  The channel sums meet by shuffles before one
+// shared-memory add per warp and channel.
+// All 17 layers of a training step at batch 8 (ncu): 460 us one pixel at a time
+// with eight shared adds a thread, 334 us so.
+template <int PX>
+__global__ void __launch_bounds__(256) dsilu_bias_kernel(const __nv_bfloat16* dy, int ldy, int yoff,
+                                                        const __nv_bfloat16* z, __nv_bfloat16* dz, long long npix, int c,
+                                                        float* db) {
   extern __shared__ float red[];  // c
   const int G = c >> 3, lanes = blockDim.x / G;
   const int g = threadIdx.x % G, pl = threadIdx.x / G;
   for (int q = threadIdx.x; q < c; q += blockDim.x) red[q] = 0.f;
   __syncthreads();
   float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  for (long long p = blockIdx.x * (long long)lanes + pl; p < npix; p += (long long)gridDim.x * lanes) {
-    float gy[8], zz[8], d[8];
-    unpack8(ld8(dy + p * ldy + yoff + 8 * g), gy);
-    unpack8(ld8(z + p * c + 8 * g), zz);
+  const long long step = (long long)gridDim.x * lanes;
+  for (long long p0 = blockIdx.x * (long long)lanes + pl; p0 < npix; p0 += PX * step) {
+    uint4 gv[PX], zv[PX];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) d[e] = gy[e] * dsilu(zz[e]);
-    const uint4 o = pack8(d);
-    st8(dz + p * c + 8 * g, o);
-    float r[8];
-    unpack8(o, r);
+    for (int k = 0; k < PX; ++k) {
+      const long long p = p0 + k * step;
+      if (p < npix) {
+        gv[k] = ld8(dy + p * ldy + yoff + 8 * g);
+        zv[k] = ld8(z + p * c + 8 * g);
+      }
+    }
 #pragma unroll
-    for (int e = 0; e < 8; ++e) s[e] += r[e];
+    for (int k = 0; k < PX; ++k) {
+      const long long p = p0 + k * step;
+      if (p < npix) {
+        float gy[8], zz[8], d[8], r[8];
+        unpack8(gv[k], gy);
+        unpack8(zv[k], zz);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) d[e] = gy[e] * dsilu(zz[e]);
+        const uint4 o = pack8(d);
+        st8(dz + p * c + 8 * g, o);
+        unpack8(o, r);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s[e] += r[e];
+      }
+    }
   }
+  // lanes of a warp that hold the same channels (G divides 32): fold them
+  const bool fold = G < 32 && 32 % G == 0 && blockDim.x % 32 == 0;
+  if (fold)
+    for (int o = 16; o >= G; o >>= 1)
 #pragma unroll
-  for (int e = 0; e < 8; ++e) atomicAdd(&red[8 * g + e], s[e]);
+      for (int e = 0; e < 8; ++e) s[e] += __shfl_xor_sync(0xffffffffu, s[e], o);
+  if (!fold || (threadIdx.x & 31) < G)
+#pragma unroll
+    for (int e = 0; e < 8; ++e) atomicAdd(&red[8 * g + e], s[e]);
   __syncthreads();
   for (int q = threadIdx.x; q < c; q += blockDim.x) atomicAdd(db + q, red[q]);
 }
@@ -356,29 +386,6 @@ __global__ void up_bwd_kernel(const __nv_bfloat16* dy, __nv_bfloat16* dx, int B,
   }
 }
 
-// copy c channels from (src, lds, soff) to (dst, ldd, doff); accumulate adds
-__global__ void copy_ch_kernel(const __nv_bfloat16* src, int lds, int soff, __nv_bfloat16* dst, int ldd, int doff,
-                               long long npix, int c, int accumulate) {
-  const int G = c >> 3;
-  const long long n = npix * G;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const long long p = i / G;
-    const int g = (int)(i - p * G);
-    const uint4 v = ld8(src + p * lds + soff + 8 * g);
-    __nv_bfloat16* d = dst + p * ldd + doff + 8 * g;
-    if (accumulate) {
-      float a[8], b[8];
-      unpack8(v, a);
-      unpack8(ld8(d), b);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) a[e] += b[e];
-      st8(d, pack8(a));
-    } else {
-      st8(d, v);
-    }
-  }
-}
-
 // FP32 NHWC (cin channels) -> normalised BF16 NHWC padded to ldo channels with zeros
 __global__ void to_bf16_kernel(const float* x, int cin, __nv_bfloat16* y, int ldo, long long npix, const Norm nm) {
   const long long n = npix * ldo;
@@ -409,84 +416,102 @@ __global__ void to_bf16_16_kernel(const float* x, int cin, __nv_bfloat16* y, lon
   }
 }
 
-// output layer: 1x1 convolution cin -> cout (cout <= 16), FP32 out, no activation, then the
+// output layer: 1x1 convolution cin -> CO (<= 16), FP32 out, no activation, then the
 // output map (scale, optional residual from the raw FP32 input xin of in_ch channels);
 // a thread takes one pixel, weights in shared memory
-__global__ void head_fwd_kernel(const __nv_bfloat16* x, int cin, const float* w, const float* b, float* y, int cout,
+template <int CO>
+__global__ void head_fwd_kernel(const __nv_bfloat16* x, int cin, const float* w, const float* b, float* y,
                                 long long npix, const float* xin, int in_ch, const Norm nm) {
-  extern __shared__ __align__(16) float sw[];  // [cout][cin], bias[cout]
-  for (int q = threadIdx.x; q < cout * cin + cout; q += blockDim.x) sw[q] = q < cout * cin ? w[q] : b[q - cout * cin];
+  extern __shared__ __align__(16) float sw[];  // [CO][cin], bias[CO]
+  for (int q = threadIdx.x; q < CO * cin + CO; q += blockDim.x) sw[q] = q < CO * cin ? w[q] : b[q - CO * cin];
   __syncthreads();
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npix; p += (long long)gridDim.x * blockDim.x) {
-    float acc[16];
+    float acc[CO];
 #pragma unroll
-    for (int o = 0; o < 16; ++o) acc[o] = o < cout ? sw[cout * cin + o] : 0.f;
+    for (int o = 0; o < CO; ++o) acc[o] = sw[CO * cin + o];
+#pragma unroll 4
     for (int c0 = 0; c0 < cin; c0 += 8) {
       float f[8];
       unpack8(ld8(x + p * cin + c0), f);
 #pragma unroll
-      for (int o = 0; o < 16; ++o) {
-        if (o < cout) {
-          const float* wr = sw + o * cin + c0;
+      for (int o = 0; o < CO; ++o) {
+        const float4* wr = reinterpret_cast<const float4*>(sw + o * cin + c0);  // cin is a multiple of 16
+        const float4 w0 = wr[0], w1 = wr[1];
+        const float ww[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
 #pragma unroll
-          for (int e = 0; e < 8; ++e) acc[o] += wr[e] * f[e];
-        }
+        for (int e = 0; e < 8; ++e) acc[o] += ww[e] * f[e];
       }
     }
 #pragma unroll
-    for (int o = 0; o < 16; ++o)
-      if (o < cout) y[p * cout + o] = (nm.residual ? xin[p * in_ch + o] : 0.f) + nm.oscale[o] * acc[o];
+    for (int o = 0; o < CO; ++o) y[p * CO + o] = (nm.residual ? xin[p * in_ch + o] : 0.f) + nm.oscale[o] * acc[o];
   }
 }
 
 // its adjoint: dX = dY W (bf16), dW += sum_p dY x^T, db += sum_p dY.  A block stages a tile
-// of TP pixels; thread t computes dX of pixel t, and each (o, c) pair of dW, db is
-// accumulated by one thread in shared memory.
-__global__ void head_bwd_kernel(const __nv_bfloat16* x, int cin, const float* w, const float* dy, int cout,
-                                __nv_bfloat16* dx, float* dw, float* db, long long npix, int TP) {
+// of TP pixels; thread t computes dX of pixel t; for dW a lane takes a channel and its
+// warp a share of the tile's pixels (a thread per (o, c) pair walked all
+// pixels)
+template <int CO>
+__global__ void __launch_bounds__(256) head_bwd_kernel(const __nv_bfloat16* x, int cin, const float* w, const float* dy,
+                                                      __nv_bfloat16* dx, float* dw, float* db, long long npix, int TP) {
   extern __shared__ __align__(16) float sh[];
-  const int npair = cout * cin + cout;
-  float* sacc = sh;                         // npair
-  float* sw = sacc + npair;                 // cout * cin
-  float* sdy = sw + cout * cin;             // TP * cout
+  const int npair = CO * cin + CO;
+  float* sw = sh;                           // CO * cin (rows of 16 bytes)
+  float* sacc = sw + CO * cin;              // npair
+  float* sdy = sacc + npair;                // TP * CO
   // the staged activations start on a 16-byte boundary (they are moved 8 channels at a time)
-  const int nf = (npair + cout * cin + TP * cout + 3) & ~3;
+  const int nf = (npair + CO * cin + TP * CO + 3) & ~3;
   __nv_bfloat16* sx = reinterpret_cast<__nv_bfloat16*>(sh + nf);   // TP * cin
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   for (int q = threadIdx.x; q < npair; q += blockDim.x) sacc[q] = 0.f;
-  for (int q = threadIdx.x; q < cout * cin; q += blockDim.x) sw[q] = w[q];
+  for (int q = threadIdx.x; q < CO * cin; q += blockDim.x) sw[q] = w[q];
+  float sb = 0.f;  // lane o < CO: its share of db[o]
   for (long long p0 = (long long)blockIdx.x * TP; p0 < npix; p0 += (long long)gridDim.x * TP) {
     const int np = (int)(npix - p0 < TP ? npix - p0 : TP);
     __syncthreads();
-    for (int q = threadIdx.x; q < np * cout; q += blockDim.x) sdy[q] = dy[p0 * cout + q];
+    for (int q = threadIdx.x; q < np * CO; q += blockDim.x) sdy[q] = dy[p0 * CO + q];
     for (int q = threadIdx.x; q < np * (cin >> 3); q += blockDim.x)
       st8(sx + q * 8, ld8(x + p0 * cin + (long long)q * 8));
     __syncthreads();
     for (int t = threadIdx.x; t < np; t += blockDim.x) {
+      float g[CO];
+#pragma unroll
+      for (int o = 0; o < CO; ++o) g[o] = sdy[t * CO + o];
       for (int c0 = 0; c0 < cin; c0 += 8) {
         float d[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int o = 0; o < cout; ++o) {
-          const float g = sdy[t * cout + o];
 #pragma unroll
-          for (int e = 0; e < 8; ++e) d[e] += g * sw[o * cin + c0 + e];
+        for (int o = 0; o < CO; ++o) {
+          const float4* wr = reinterpret_cast<const float4*>(sw + o * cin + c0);
+          const float4 w0 = wr[0], w1 = wr[1];
+          const float ww[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+#pragma unroll
+          for (int e = 0; e < 8; ++e) d[e] += g[o] * ww[e];
         }
         st8(dx + (p0 + t) * cin + c0, pack8(d));
       }
     }
-    for (int q = threadIdx.x; q < npair; q += blockDim.x) {
-      float acc = 0.f;
-      if (q < cout * cin) {
-        const int o = q / cin, c = q - o * cin;
-        for (int t = 0; t < np; ++t) acc += sdy[t * cout + o] * __bfloat162float(sx[t * cin + c]);
-      } else {
-        const int o = q - cout * cin;
-        for (int t = 0; t < np; ++t) acc += sdy[t * cout + o];
-      }
-      sacc[q] += acc;
+    for (int c0 = 0; c0 < cin; c0 += 32) {
+      const int c = c0 + lane;
+      float acc[CO];
+#pragma unroll
+      for (int o = 0; o < CO; ++o) acc[o] = 0.f;
+      if (c < cin)
+        for (int t = warp; t < np; t += nwarp) {
+          const float xv = __bfloat162float(sx[t * cin + c]);
+#pragma unroll
+          for (int o = 0; o < CO; ++o) acc[o] += sdy[t * CO + o] * xv;
+        }
+      if (c < cin)
+#pragma unroll
+        for (int o = 0; o < CO; ++o) atomicAdd(&sacc[o * cin + c], acc[o]);
     }
+    if (lane < CO)
+      for (int t = warp; t < np; t += nwarp) sb += sdy[t * CO + lane];
   }
+  if (lane < CO) atomicAdd(&sacc[CO * cin + lane], sb);
   __syncthreads();
-  for (int q = threadIdx.x; q < cout * cin; q += blockDim.x) atomicAdd(dw + q, sacc[q]);
-  for (int q = threadIdx.x; q < cout; q += blockDim.x) atomicAdd(db + q, sacc[cout * cin + q]);
+  for (int q = threadIdx.x; q < CO * cin; q += blockDim.x) atomicAdd(dw + q, sacc[q]);
+  for (int q = threadIdx.x; q < CO; q += blockDim.x) atomicAdd(db + q, sacc[CO * cin + q]);
 }
 
 // mean squared error of the scaled output error e = (y - t) / oscale and its gradient with
@@ -523,26 +548,48 @@ __global__ void adam_kernel(float* w, const float* gr, float* m, float* v, long 
   }
 }
 
-// WT (FP32 master, [co][tap*cin + ci]) -> BF16 WT and its transpose WD [ci][tap*cout + co]
-// The BF16 copies of a convolution's weights w[co][tap][ci]: wt in the same
+// The BF16 copies of the convolutions' weights w[co][tap][ci]: wt in the same
 // order, wd transposed for the data gradient ([ci][tap][co]), and for the
 // tcgen05 kernels wtp / wdp (either may be NULL) packed per K chunk of 16
 // channels as [chunk][tap][half][n][8], n the output channel of the product
 // (co for the forward, ci for the data gradient) and the 8 channels of the
 // half contiguous: the weights of a chunk for a block of n are 18 runs of
-// 16-byte rows, one box of one bulk tensor copy.
-__global__ void weights_bf16_kernel(const float* w, __nv_bfloat16* wt, __nv_bfloat16* wd, __nv_bfloat16* wtp,
-                                    __nv_bfloat16* wdp, int cout, int cin, int taps) {
-  const long long n = (long long)cout * taps * cin;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int co = (int)(i / ((long long)taps * cin));
-    const int k = (int)(i - (long long)co * taps * cin);
-    const int tap = k / cin, ci = k - tap * cin;
-    const __nv_bfloat16 b = __float2bfloat16_rn(w[i]);
-    wt[i] = b;
-    if (wd) wd[((size_t)ci * taps + tap) * cout + co] = b;
-    if (wtp) wtp[(((size_t)(ci >> 4) * 18 + tap * 2 + ((ci >> 3) & 1)) * cout + co) * 8 + (ci & 7)] = b;
-    if (wdp) wdp[(((size_t)(co >> 4) * 18 + tap * 2 + ((co >> 3) & 1)) * cin + ci) * 8 + (co & 7)] = b;
+// 16-byte rows.  All layers in one launch; a thread moves one 16-byte row: first
+// the rows along ci (wt, wtp), then those along co (wd, wdp), in the order
+// of the packed form so that its stores are contiguous.  (A launch per layer, an
+// element per thread: 96 us of a training step; 15 us so.)
+__global__ void __launch_bounds__(256) weights_bf16_kernel(const WeightLayers ls) {
+  for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < ls.rows; u += (long long)gridDim.x * blockDim.x) {
+    const bool fwd = u < ls.rows / 2;
+    const long long v = fwd ? u : u - ls.rows / 2;
+    int li = 0;
+    while (li + 1 < ls.n && v >= ls.l[li + 1].first) ++li;
+    const WeightLayer& l = ls.l[li];
+    // row k of the packed order: [chunk][tap][half][n]
+    const int nn = fwd ? l.cout : l.cin;
+    long long k = v - l.first;
+    const int n = (int)(k % nn);
+    k /= nn;
+    const int half = (int)(k & 1);
+    k >>= 1;
+    const int tap = (int)(k % l.taps), c0 = (int)(k / l.taps) * 16 + half * 8;
+    float f[8];
+    if (fwd) {
+      const float* src = l.w + ((size_t)n * l.taps + tap) * l.cin + c0;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) f[e] = src[e];
+    } else {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) f[e] = l.w[((size_t)(c0 + e) * l.taps + tap) * l.cin + n];
+    }
+    uint4 o;
+    __nv_bfloat16* h = reinterpret_cast<__nv_bfloat16*>(&o);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) h[e] = __float2bfloat16_rn(f[e]);
+    __nv_bfloat16* plain = fwd ? l.wt : l.wd;
+    __nv_bfloat16* packed = fwd ? l.wtp : l.wdp;
+    st8(plain + ((size_t)n * l.taps + tap) * (fwd ? l.cin : l.cout) + c0, o);
+    if (packed) st8(packed + (size_t)(v - l.first) * 8, o);
   }
 }
 
@@ -586,9 +633,9 @@ cudaError_t dsilu_bias(const __nv_bfloat16* dy, int ldy, int yoff, const __nv_bf
                        long long npix, int c, float* db, cudaStream_t s) {
   const int G = c / 8;
   const int lanes = G >= 256 ? 1 : 256 / G;
-  long long nb = (npix + lanes - 1) / lanes;
-  if (nb > 152 * 8) nb = 152 * 8;
-  dsilu_bias_kernel<<<(unsigned)nb, G * lanes, c * sizeof(float), s>>>(dy, ldy, yoff, z, dz, npix, c, db);
+  long long nb = (npix + 2LL * lanes - 1) / (2 * lanes);
+  if (nb > 152 * 6) nb = 152 * 6;
+  dsilu_bias_kernel<2><<<(unsigned)nb, G * lanes, c * sizeof(float), s>>>(dy, ldy, yoff, z, dz, npix, c, db);
   return cudaGetLastError();
 }
 
@@ -609,12 +656,6 @@ cudaError_t up_bwd(const __nv_bfloat16* dy, __nv_bfloat16* dx, int B, int H, int
   return cudaGetLastError();
 }
 
-cudaError_t copy_ch(const __nv_bfloat16* src, int lds, int soff, __nv_bfloat16* dst, int ldd, int doff, long long npix,
-                    int c, int accumulate, cudaStream_t s) {
-  copy_ch_kernel<<<blocks_for(npix * c / 8), 256, 0, s>>>(src, lds, soff, dst, ldd, doff, npix, c, accumulate);
-  return cudaGetLastError();
-}
-
 cudaError_t to_bf16(const float* x, int cin, __nv_bfloat16* y, int ldo, long long npix, const Norm& nm,
                     cudaStream_t s) {
   if (ldo == 16 && cin <= 16 && (reinterpret_cast<uintptr_t>(y) & 15) == 0)
@@ -624,11 +665,23 @@ cudaError_t to_bf16(const float* x, int cin, __nv_bfloat16* y, int ldo, long lon
   return cudaGetLastError();
 }
 
+#define GPE2P_HEAD_SWITCH(F)                                                                                   \
+  switch (cout) {                                                                                             \
+    case 1: return F(1); case 2: return F(2); case 3: return F(3); case 4: return F(4);                       \
+    case 5: return F(5); case 6: return F(6); case 7: return F(7); case 8: return F(8);                       \
+    case 9: return F(9); case 10: return F(10); case 11: return F(11); case 12: return F(12);                 \
+    case 13: return F(13); case 14: return F(14); case 15: return F(15); default: return F(16);               \
+  }
+
 cudaError_t head_fwd(const __nv_bfloat16* x, int cin, const float* w, const float* b, float* y, int cout,
                      long long npix, const float* xin, int in_ch, const Norm& nm, cudaStream_t s) {
-  head_fwd_kernel<<<blocks_for(npix), 256, (cout * cin + cout) * sizeof(float), s>>>(x, cin, w, b, y, cout, npix,
-                                                                                      xin, in_ch, nm);
-  return cudaGetLastError();
+  auto go = [&](auto k) {
+    k<<<blocks_for(npix), 256, (cout * cin + cout) * sizeof(float), s>>>(x, cin, w, b, y, npix, xin, in_ch, nm);
+    return cudaGetLastError();
+  };
+#define GPE2P_HF(N) go(head_fwd_kernel<N>)
+  GPE2P_HEAD_SWITCH(GPE2P_HF)
+#undef GPE2P_HF
 }
 
 cudaError_t head_bwd(const __nv_bfloat16* x, int cin, const float* w, const float* dy, int cout, __nv_bfloat16* dx,
@@ -640,12 +693,17 @@ cudaError_t head_bwd(const __nv_bfloat16* x, int cin, const float* w, const floa
   const size_t smem = nf * sizeof(float) + (size_t)TP * cin * 2;
   long long nb = (npix + TP - 1) / TP;
   if (nb > 152 * 4) nb = 152 * 4;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(head_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  head_bwd_kernel<<<(unsigned)nb, 256, smem, s>>>(x, cin, w, dy, cout, dx, dw, db, npix, TP);
-  return cudaGetLastError();
+  auto go = [&](auto k) {
+    if (smem > 48 * 1024) {
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+    }
+    k<<<(unsigned)nb, 256, smem, s>>>(x, cin, w, dy, dx, dw, db, npix, TP);
+    return cudaGetLastError();
+  };
+#define GPE2P_HB(N) go(head_bwd_kernel<N>)
+  GPE2P_HEAD_SWITCH(GPE2P_HB)
+#undef GPE2P_HB
 }
 
 cudaError_t mse(const float* y, const float* t, float* dy, long long n, int cout, const Norm& nm, float* loss,
@@ -660,11 +718,8 @@ cudaError_t adam(float* w, const float* g, float* m, float* v, long long n, floa
   return cudaGetLastError();
 }
 
-cudaError_t weights_bf16(const float* w, __nv_bfloat16* wt, __nv_bfloat16* wd, __nv_bfloat16* wtp,
-                         __nv_bfloat16* wdp, int cout, int cin, int taps, cudaStream_t s) {
-  const bool packable = taps == 9 && cin % 16 == 0 && cout % 16 == 0;
-  weights_bf16_kernel<<<blocks_for((long long)cout * cin * taps), 256, 0, s>>>(
-      w, wt, wd, packable ? wtp : nullptr, packable ? wdp : nullptr, cout, cin, taps);
+cudaError_t weights_bf16(const WeightLayers& ls, cudaStream_t s) {
+  weights_bf16_kernel<<<blocks_for(ls.rows), 256, 0, s>>>(ls);
   return cudaGetLastError();
 }
 

@@ -62,8 +62,6 @@ cudaError_t pool_fwd(const __nv_bfloat16* x, int ldx, int xoff, __nv_bfloat16* y
 cudaError_t pool_bwd(const __nv_bfloat16* dy, __nv_bfloat16* dx, int ldx, int xoff, int B, int H, int W, int c,
                      int accumulate, cudaStream_t s);
 cudaError_t up_bwd(const __nv_bfloat16* dy, __nv_bfloat16* dx, int B, int H, int W, int c, cudaStream_t s);
-cudaError_t copy_ch(const __nv_bfloat16* src, int lds, int soff, __nv_bfloat16* dst, int ldd, int doff,
-                    long long npix, int c, int accumulate, cudaStream_t s);
 cudaError_t to_bf16(const float* x, int cin, __nv_bfloat16* y, int ldo, long long npix, const Norm& nm,
                     cudaStream_t s);
 cudaError_t head_fwd(const __nv_bfloat16* x, int cin, const float* w, const float* b, float* y, int cout,
@@ -74,8 +72,20 @@ cudaError_t mse(const float* y, const float* t, float* dy, long long n, int cout
                 cudaStream_t s);
 cudaError_t adam(float* w, const float* g, float* m, float* v, long long n, float lr, float b1, float b2, float eps,
                  float c1, float c2, cudaStream_t s);
-cudaError_t weights_bf16(const float* w, __nv_bfloat16* wt, __nv_bfloat16* wd, __nv_bfloat16* wtp,
-                         __nv_bfloat16* wdp, int cout, int cin, int taps, cudaStream_t s);
+// the convolutions whose BF16 copies weights_bf16 refreshes: FP32 weights, the copies (the
+// packed ones NULL unless taps is 9), and the layer's first 16-byte row in each direction
+struct WeightLayer {
+  const float* w;
+  __nv_bfloat16 *wt, *wd, *wtp, *wdp;
+  int cout, cin, taps;
+  long long first;
+};
+struct WeightLayers {
+  WeightLayer l[32];
+  int n;
+  long long rows;  // of all layers, both directions
+};
+cudaError_t weights_bf16(const WeightLayers& ls, cudaStream_t s);
 
 }  // namespace nn
 }  // namespace gpe2p
