@@ -599,14 +599,15 @@ cudaError_t conv3_tc(const ConvArgs& a, cudaStream_t s) {
 //          the tile overhangs the image.
 // 3 MMAs (6 for CIB = 64) per K step in place of one per tap; the
 // accumulators of all taps stay in tensor memory over all tiles of the CTA
-// (at most 384 columns), which then adds them to dW with FP32 reductions
+// (at most 384 of 512 columns), which then adds them to dW with FP32 reductions
 // coalesced over ci.
 //
-// Bound: the MMA issue and operand rate (40 to 53 cycles per MMA whatever N <= 64),
-// not memory.  All layers of a training step of the 256 x 256, batch 8,
-// 32-64-128-256 net: 0.55 ms (17 launches), 5.41 ms on the mma.sync kernel,
-// which transposes both operands element by element on their way to shared
-// memory; the training step 2.34 against 7.18 ms.
+// Bound: the copies and the MMAs of a tile take nearly the same time beside each
+// other, and the final reductions follow.  All layers of a training step of the
+// 256 x 256, batch 8, 32-64-128-256 net: 0.50 ms (17 launches); without the
+// reductions or with an eighth of the MMAs each 0.45 ms, without the copies 0.48 ms;
+// 5.41 ms on the mma.sync kernel, which transposes both operands element by
+// element on their way to shared memory.
 constexpr int WG_PROD = 128;              // producer threads (warps 0-3, then the epilogue)
 constexpr int WG_NTHR = WG_PROD + 32;     // warp 4 issues the MMAs
 constexpr int WG_SMAX = 6;
@@ -615,11 +616,16 @@ template <int CIB, int COB>
 struct WgCfg {
   static constexpr int CG = CIB / 8, OG = COB / 8;
   static constexpr int X_BYTES = WH * CG * WW * 16;
-  static constexpr int Z_BYTES = OG * TH * TW * 16;
+  // dZ rows per 8-channel group, one more than its pixels: consecutive threads
+  // write consecutive groups of a pixel, and 2048 bytes apart they would all hit
+  // the same banks
+  static constexpr int ZR = TH * TW + 1;
+  static constexpr int Z_BYTES = OG * ZR * 16;
   static constexpr int STAGE = X_BYTES + Z_BYTES;
   static constexpr int MB = CIB == 64 ? 2 : 1;        // MMAs of M = 128 per dx
   static constexpr int COLS = 3 * MB * COB;
   static constexpr int TCOLS = COLS <= 64 ? 64 : (COLS <= 128 ? 128 : (COLS <= 256 ? 256 : 512));
+  static_assert(COLS <= 512, "the accumulators of all taps fit in tensor memory");
   // the last rows of M read past the window's rows: into the stage's dZ
   static_assert((TH - 1 + 128 * MB / CIB) * CG * WW * 16 <= STAGE, "the operand's overhang stays inside the stage");
 };
@@ -706,7 +712,7 @@ __global__ void __launch_bounds__(WG_NTHR) wgrad3_tc_kernel(const ConvArgs a, in
         const int r = zr + ZP * j;
         const int y = tg.y0 + r / TW, x = tg.x0 + r % TW;
         const bool valid = y < H && x < W;
-        cp_async16_zfill(Z + (zg * TH * TW + r) * 16,
+        cp_async16_zfill(Z + (zg * C::ZR + r) * 16,
                          zsrc + (valid ? ((size_t)(tg.b * H + y) * W + x) * a.ldz : (size_t)0), valid);
       }
       cp_async_arrive_noinc(&full[s]);
@@ -746,7 +752,7 @@ __global__ void __launch_bounds__(WG_NTHR) wgrad3_tc_kernel(const ConvArgs a, in
     // ---- the MMA issuer ----
     // both operands MN-major (bits 15 and 16)
     const uint32_t idesc = idesc_bf16<COB>() | (1u << 15) | (1u << 16);
-    const uint64_t ad_lay = sdesc(0, C::CG * WW * 16, WW * 16), bd_lay = sdesc(0, 128, TH * TW * 16);
+    const uint64_t ad_lay = sdesc(0, C::CG * WW * 16, WW * 16), bd_lay = sdesc(0, 128, C::ZR * 16);
     const uint32_t base = smem_u32(stages);
     bool ok = true;
     int s = 0;
@@ -804,7 +810,7 @@ cudaError_t launch_wgrad(const ConvArgs& a, cudaStream_t s) {
   // reach one MMA per 40 cycles, one thread one per 53), and as many stages
   // as fit beside each other
   const int occ = C::TCOLS <= 256 ? 2 : 1;
-  int ns = (occ == 2 ? 108 * 1024 : SMEM_MAX) / C::STAGE;
+  int ns = (occ == 2 ? 108 * 1024 : SMEM_MAX - 1024 - HEAD) / C::STAGE;
   if (ns > WG_SMAX) ns = WG_SMAX;
   const int smem = 1024 + HEAD + ns * C::STAGE;
   const int gy = a.cin / CIB, gz = a.cout / COB;
@@ -845,7 +851,13 @@ bool conv_wgrad_tc_supported(const ConvArgs& a) {
          ((reinterpret_cast<uintptr_t>(a.x) | reinterpret_cast<uintptr_t>(a.dz)) & 15) == 0;
 }
 
+// The blocks of channels: N = COB = 128 where cout allows it, because three MMAs of
+// 32 x 128 weights replace six of 64 x 64 in a K step of all taps; CIB is then 32,
+// so that the accumulators of three column shifts fit in tensor memory.  256 -> 128
+// channels at 64 x 64, batch 8: 41 us at 64 x 64, 37 us at 32 x 128, 34 us with
+// dZ's groups off each other's banks as well.
 cudaError_t conv_wgrad_tc(const ConvArgs& a, cudaStream_t s) {
+  if (a.cout % 128 == 0 && a.cin % 32 == 0) return launch_wgrad<32, 128>(a, s);
   if (a.cin % 64 == 0) return wgrad_co<64>(a, s);
   if (a.cin % 32 == 0) return wgrad_co<32>(a, s);
   return wgrad_co<16>(a, s);

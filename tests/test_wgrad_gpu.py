@@ -1,6 +1,6 @@
 """The tcgen05 weight gradient at the shapes where its tiling can go wrong:
 images smaller than its 16 x 8 pixel tile, images the tiles overhang, channel
-counts that take each of its block sizes (16, 32, 64, and 48 = 3 x 16), the
+counts that take each of its block sizes (16, 32, 64, 128, and 48 = 3 x 16), the
 upsampled input of the decoder, and more tiles than CTAs.
 
 Both sides take the same BF16 activations and dZ (the network oracle with
@@ -19,7 +19,8 @@ from paper_2011_00814_gb300 import build, gpe2p
 pytestmark = pytest.mark.gpu
 
 SHAPES = [(1, [16], 1, 1, 1), (1, [64], 17, 9, 2), (2, [16, 32], 6, 10, 3), (2, [32, 64], 34, 14, 1),
-          (2, [48, 96], 18, 26, 2), (2, [64, 128], 32, 8, 2), (3, [32, 16, 64], 36, 20, 1), (1, [32], 200, 136, 3)]
+          (2, [48, 96], 18, 26, 2), (2, [64, 128], 32, 8, 2), (3, [32, 16, 64], 36, 20, 1), (1, [32], 200, 136, 3),
+          (2, [32, 128], 20, 12, 2), (2, [128, 256], 18, 14, 1)]
 
 
 @pytest.mark.parametrize("levels,channels,h,w,b", SHAPES)
