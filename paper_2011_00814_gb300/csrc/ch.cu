@@ -16,13 +16,15 @@ template <typename real, int TXv, int TYv, int CPT>
 __global__ void __launch_bounds__(TXv* TYv / CPT) ch2d_kernel(const __grid_constant__ KParams<real> P,
                                                           const CHArgs<real> A) {
   extern __shared__ __align__(16) unsigned char smraw2d[];
+  after_previous_kernel();
   ch2d_tile<real, TXv, TYv, CPT>(P, A, blockIdx.x * TXv, blockIdx.y * TYv, reinterpret_cast<real*>(smraw2d));
 }
 
 template <typename real, int TXv, int TYv, int CPT>
 __global__ void __launch_bounds__(TXv* TYv / CPT) mu2d_kernel(const __grid_constant__ KParams<real> P,
-                                                          const real* __restrict__ phi, real* __restrict__ mu) {
+                                                          const real* phi, real* mu) {
   __shared__ real sm[(TXv + 2) * (TYv + 2)];
+  after_previous_kernel();
   mu2d_tile<real, TXv, TYv, CPT>(P, phi, mu, blockIdx.x * TXv, blockIdx.y * TYv, sm);
 }
 
@@ -38,15 +40,13 @@ static cudaError_t ch2d_go(const KParams<real>& P, const CHArgs<real>& A, cudaSt
   constexpr size_t sm = sizeof(real) * (size_t)C_N * (TXv + 2) * (TYv + 2);
   static_assert(sm <= 48 * 1024, "no opt-in shared memory");
   const dim3 grd((P.n[0] + TXv - 1) / TXv, (P.n[1] + TYv - 1) / TYv);
-  ch2d_kernel<real, TXv, TYv, CPT><<<grd, TXv * TYv / CPT, sm, s>>>(P, A);
-  return cudaGetLastError();
+  return launch_step(ch2d_kernel<real, TXv, TYv, CPT>, small_grid(P), grd, TXv * TYv / CPT, sm, s, P, A);
 }
 
 template <typename real, int TXv, int TYv, int CPT>
 static cudaError_t mu2d_go(const KParams<real>& P, const real* phi, real* mu, cudaStream_t s) {
   const dim3 grd((P.n[0] + TXv - 1) / TXv, (P.n[1] + TYv - 1) / TYv);
-  mu2d_kernel<real, TXv, TYv, CPT><<<grd, TXv * TYv / CPT, 0, s>>>(P, phi, mu);
-  return cudaGetLastError();
+  return launch_step(mu2d_kernel<real, TXv, TYv, CPT>, small_grid(P), grd, TXv * TYv / CPT, 0, s, P, phi, mu);
 }
 
 // ---------------------------------------------------------------------------

@@ -26,6 +26,7 @@ template <int MODE, int TXv, int TYv, int NT>
 __global__ void __launch_bounds__(NT) flow2d64_kernel(const __grid_constant__ KParams<double> P,
                                                      const FlowArgs<double> A) {
   extern __shared__ __align__(16) double sm2d64[];
+  after_previous_kernel();
   flow2d_tile64<MODE, TXv, TYv, NT>(P, A, blockIdx.x * TXv, blockIdx.y * TYv, sm2d64);
 }
 
@@ -34,23 +35,23 @@ static cudaError_t flow64_go(const KParams<double>& P, const FlowArgs<double>& A
   static_assert(flow64_smem<TXv, TYv>(0) <= 48 * 1024, "no opt-in shared memory");
   const size_t sm = flow64_smem<TXv, TYv>(mode);
   const dim3 grd((P.n[0] + TXv - 1) / TXv, (P.n[1] + TYv - 1) / TYv);
-  if (mode == 0) flow2d64_kernel<0, TXv, TYv, NT><<<grd, NT, sm, s>>>(P, A);
-  else if (mode == 1) flow2d64_kernel<1, TXv, TYv, NT><<<grd, NT, sm, s>>>(P, A);
-  else flow2d64_kernel<2, TXv, TYv, NT><<<grd, NT, sm, s>>>(P, A);
-  return cudaGetLastError();
+  return launch_step(mode == 0 ? flow2d64_kernel<0, TXv, TYv, NT>
+                               : (mode == 1 ? flow2d64_kernel<1, TXv, TYv, NT> : flow2d64_kernel<2, TXv, TYv, NT>),
+                     small_grid(P), grd, NT, sm, s, P, A);
 }
 
 // The tile of a 2D FP64 stage: 32 x 8 where two tiles fall on every SM, else a
 // smaller one, since a small grid is bound by the FP64 operations of its
 // busiest SM (64 x 64: 16 tiles of 32 x 8 or 128 of 8 x 4).
 // Measured: 20 steps of 64 x 64 with host arrays in and out 1.73 -> 0.80 ms,
-// 50 steps of 128 x 64 4.05 -> 1.56 ms (32 x 8 tiles of FlowOps before).
+// 50 steps of 128 x 64 4.05 -> 1.56 ms (32 x 8 tiles of FlowOps before); with
+// overlapped launches 0.74 and 1.43 ms.
 static cudaError_t flow64(const KParams<double>& P, const FlowArgs<double>& A, int mode, cudaStream_t s) {
   auto tiles = [&](int tx, int ty) {
     return (long long)((P.n[0] + tx - 1) / tx) * ((P.n[1] + ty - 1) / ty);
   };
   if (tiles(32, 8) >= 2 * 152) return flow64_go<32, 8, 256>(P, A, mode, s);
-  if (tiles(16, 4) >= 2 * 152) return flow64_go<16, 4, 192>(P, A, mode, s);
+  if (!small_grid(P)) return flow64_go<16, 4, 192>(P, A, mode, s);
   return flow64_go<8, 4, 96>(P, A, mode, s);
 }
 

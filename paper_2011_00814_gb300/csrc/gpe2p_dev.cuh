@@ -12,6 +12,19 @@
 
 namespace gpe2p {
 
+// Kernels of a 2D step can be programmatic dependents of each other
+// (launch_step, gpe2p_launch.h): their blocks are placed while the kernel before
+// them runs.  Every thread waits for that kernel's end before its first access to
+// global memory, and lets the next kernel's blocks be placed only then; so a kernel
+// ends after all before it, and no more than one waits beside a running one.
+// Pointers of such a kernel's own arguments carry no __restrict__: a load the
+// compiler knows to be invariant could move above the wait.
+__device__ __forceinline__ void after_previous_kernel() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+
 enum { BC_PERIODIC = 0, BC_NOSLIP = 1, BC_FREESLIP = 2 };
 
 // Tile of one thread block: TX x TY cells in (x, y); 3D kernels march the tile

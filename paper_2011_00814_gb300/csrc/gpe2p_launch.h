@@ -2,12 +2,47 @@
 // (internal to the library; the public interface is include/gpe2p.h).
 #pragma once
 
+#include <utility>
 #include <cuda_runtime.h>
 
 #include "gpe2p_dev.cuh"
 #include "ring3d.cuh"
 
 namespace gpe2p {
+
+// Launch a kernel of a 2D step, where overlap is set as the programmatic dependent of
+// the one before it on the stream (after_previous_kernel, gpe2p_dev.cuh).
+//
+// Blocks placed early gather on the SMs that are free first.  That costs nothing where
+// blocks are many and short or the grid leaves SMs free, and unbalances a grid of
+// about one wave of long blocks.  Microseconds per step, plain launches and overlapped:
+//   fused FP32 passes   128^2 8.2, 7.5   256^2 10.1, 9.6   512^2 21.0, 20.4   2048^2 228, 227
+//   FP64 stages         64^2 26.7, 25.5  128^2 34.1, 32.0  176^2 47.2, 46.7  208^2 56, 81   384^2 143, 206
+//   3D stages           101 x 75 x 130 FP32 222, 232   64 x 48 x 80 FP64 945, 1038
+// so the fused passes always overlap, the other 2D stages on small grids (small_grid),
+// the 3D stages never.
+template <class... P, class... A>
+inline cudaError_t launch_step(void (*k)(P...), bool overlap, dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                               A&&... a) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, std::forward<A>(a)...);
+}
+
+// A 2D grid with fewer than two 16 x 4 tiles per SM
+template <typename real>
+inline bool small_grid(const KParams<real>& P) {
+  return (long long)((P.n[0] + 15) / 16) * ((P.n[1] + 3) / 4) < 2 * 152;
+}
+
 
 // 3D ring kernels (flow stage, CH stage, mu): each thread computes two cells
 // adjacent in y, so a block of TX x T threads has a tile of 2T rows and

@@ -7,6 +7,7 @@ template <int NW, int R, bool AXI>
 __global__ void __launch_bounds__(32 * NW, flow_blocks(NW, R))
     flow2d_fused_kernel(const __grid_constant__ KParams<float> P, const FlowStepArgs<float> A) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  after_previous_kernel();
   flow2d_fused_tile<float, NW, R, AXI>(P, A, blockIdx.x * FUSED_X, blockIdx.y * flow_rows(NW * R),
                                        reinterpret_cast<float*>(smraw));
 }
@@ -15,6 +16,7 @@ template <int NW, int R>
 __global__ void __launch_bounds__(32 * NW, ch_blocks(NW, R))
     ch2d_fused_kernel(const __grid_constant__ KParams<float> P, const CHStepArgs<float> A) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  after_previous_kernel();
   ch2d_fused_tile<float, NW, R>(P, A, blockIdx.x * FUSED_X, blockIdx.y * ch_rows(NW * R),
                                 reinterpret_cast<float*>(smraw));
 }
@@ -25,9 +27,8 @@ static cudaError_t flow_go(const KParams<float>& P, const FlowStepArgs<float>& A
   static_assert(sm <= 48 * 1024, "no opt-in shared memory");
   constexpr int TYf = flow_rows(NW * R);
   const dim3 grd((P.n[0] + FUSED_X - 1) / FUSED_X, (P.n[1] + TYf - 1) / TYf);
-  if (P.axisym) flow2d_fused_kernel<NW, R, true><<<grd, 32 * NW, sm, s>>>(P, A);
-  else flow2d_fused_kernel<NW, R, false><<<grd, 32 * NW, sm, s>>>(P, A);
-  return cudaGetLastError();
+  return launch_step(P.axisym ? flow2d_fused_kernel<NW, R, true> : flow2d_fused_kernel<NW, R, false>, true, grd,
+                     32 * NW, sm, s, P, A);
 }
 
 template <int NW, int R>
@@ -36,8 +37,7 @@ static cudaError_t ch_go(const KParams<float>& P, const CHStepArgs<float>& A, cu
   static_assert(sm <= 48 * 1024, "no opt-in shared memory");
   constexpr int TYc = ch_rows(NW * R);
   const dim3 grd((P.n[0] + FUSED_X - 1) / FUSED_X, (P.n[1] + TYc - 1) / TYc);
-  ch2d_fused_kernel<NW, R><<<grd, 32 * NW, sm, s>>>(P, A);
-  return cudaGetLastError();
+  return launch_step(ch2d_fused_kernel<NW, R>, true, grd, 32 * NW, sm, s, P, A);
 }
 
 cudaError_t launch_flow_fused(const KParams<float>& P, const FlowStepArgs<float>& A, cudaStream_t s) {
