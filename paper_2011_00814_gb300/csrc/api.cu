@@ -1,6 +1,7 @@
 // api.cu -- host side of the C ABI declared in include/gpe2p.h: parameter
 // validation, explicit stability limits, device state, the step as a
 // sequence of kernels captured into CUDA graphs, host I/O and diagnostics.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -649,11 +650,26 @@ extern "C" int gpe2p_create(const gpe2p_params* p, void* stream, gpe2p_handle* o
   // the kc in [4, 64] that minimises waves x (kc + 2), the time of the slowest
   // SM.  Resident blocks per SM (registers and shared memory, as ncu reports
   // them): flow stage FLOW_MINB, CH stage CH_RESIDENT, mu MU_RESIDENT.
+  //
+  // CH stage and mu on a grid of at most two waves of marches of four planes: kc
+  // from 2, with r blocks resident of the very kernel (3 of the CH stage in FP64
+  // conservative form), b blocks on the busiest SM, and the last wave counted by its
+  // part of r, at least 0.8 and 0.7 of a wave, since a few blocks do not fill the
+  // SM.  kc is at most 20 and 6, and 4 for the CH stage's ring of five fields in FP32.
+  // From sweeps of kc over 20 grids.  With the rule above, and with this one, us
+  // a step:
+  //   FP32                31 x 33 x 40 93, 76   64^3 106, 92   101 x 75 x 130 202, 193
+  //   FP64 conservative   32^3 669, 505   40 x 56 x 100 1457, 1318   96^3 3427, 3413
+  // (On larger grids it gained 1 to 5 % on some and lost as much on others: there long
+  // marches save memory traffic.)
   if (h->prm.dim == 3) {
     int nsm = 152;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->dev);
+    auto columns = [&](int cols, int rows) {
+      return (long long)((h->prm.nx + cols - 1) / cols) * ((h->prm.ny + rows - 1) / rows);
+    };
     auto pick = [&](int per_sm, int cols, int rows) {
-      const long long bxy = (long long)((h->prm.nx + cols - 1) / cols) * ((h->prm.ny + rows - 1) / rows);
+      const long long bxy = columns(cols, rows);
       const long long slots = (long long)per_sm * nsm;
       long long best_kc = 4, best = -1;
       for (long long kc = 4; kc <= 64 && kc <= h->prm.nz; ++kc) {
@@ -663,9 +679,30 @@ extern "C" int gpe2p_create(const gpe2p_params* p, void* stream, gpe2p_handle* o
       }
       return (int)(best_kc > h->prm.nz ? h->prm.nz : best_kc);
     };
+    auto pick_small = [&](int usual, int r, int cols, int rows, int most, double least) {
+      const long long bxy = columns(cols, rows);
+      if (r < 1 || bxy * ((h->prm.nz + 3) / 4) > 2LL * r * nsm) return usual;
+      int best_kc = usual;
+      double best = -1;
+      for (int kc = 2; kc <= most && kc <= h->prm.nz; ++kc) {
+        const long long nb = bxy * ((h->prm.nz + kc - 1) / kc);
+        const long long b = (nb + nsm - 1) / nsm, rem = b % r;
+        const double cost = ((double)(b / r) + (rem ? std::max((double)rem / r, least) : 0.0)) * (kc + 2);
+        if (best < 0 || cost < best) { best = cost; best_kc = kc; }
+      }
+      return best_kc;
+    };
+    int rch = 0, rmu = 0;
+    const bool cons = h->prm.ch_advection != 0;
+    e = h->esize == 4 ? ch3d_resident<float>(h->prm.iso, cons, &rch, &rmu)
+                      : ch3d_resident<double>(h->prm.iso, cons, &rch, &rmu);
+    if (e != cudaSuccess) {
+      gpe2p_destroy(h);
+      return fail(nullptr, GPE2P_ECUDA, std::string("set-up: ") + cudaGetErrorString(e));
+    }
     h->kchunk = pick(h->esize == 4 ? FLOW_MINB : FLOW_MINB64, FLOW_K3_TX, FLOW_K3_TY);
-    h->kchunk_ch = pick(CH_RESIDENT, TX, CH_K3_TY);
-    h->kchunk_mu = pick(MU_RESIDENT, TX, MU_K3_TY);
+    h->kchunk_ch = pick_small(pick(CH_RESIDENT, TX, CH_K3_TY), rch, TX, CH_K3_TY, cons && h->esize == 4 ? 4 : 20, 0.8);
+    h->kchunk_mu = pick_small(pick(MU_RESIDENT, TX, MU_K3_TY), rmu, TX, MU_K3_TY, 6, 0.7);
   } else {
     h->kchunk = h->kchunk_ch = h->kchunk_mu = 1;
   }

@@ -520,6 +520,36 @@ cudaError_t launch_center_velocity(const KParams<real>& P, const real* const u0[
   return cudaGetLastError();
 }
 
+// The blocks of the 3D CH stage (the form most stages of a step run) and of mu that
+// an SM holds
+template <typename real, int ISO>
+static cudaError_t resident_go(bool conservative, int* ch, int* mu) {
+  constexpr int RING = ch_ring<real>();
+  auto ask = [](auto k, int threads, size_t sm, int* n) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k, threads, sm);
+  };
+  cudaError_t e =
+      conservative
+          ? ask(ch3d_kernel<real, ISO, 1, RING, false, false, false>, CH_NTHR,
+                ring_smem_bytes<real, 5, 0, RING, CH_K3_SY>(), ch)
+          : ask(ch3d_kernel<real, ISO, 0, RING, false, true, false>, CH_NTHR,
+                ring_smem_bytes<real, 2, 0, RING, CH_K3_SY>() + sizeof(real) * (size_t)2 * CP_N * CP_PT, ch);
+  if (e != cudaSuccess) return e;
+  return ask(mu3d_kernel<real, ISO, RING>, MU_NTHR, ring_smem_bytes<real, 1, 0, RING, MU_K3_SY>(), mu);
+}
+
+template <typename real>
+cudaError_t ch3d_resident(int iso, bool conservative, int* ch, int* mu) {
+  switch (iso) {
+    case 15: return resident_go<real, 15>(conservative, ch, mu);
+    case 19: return resident_go<real, 19>(conservative, ch, mu);
+    default: return resident_go<real, 27>(conservative, ch, mu);
+  }
+}
+template cudaError_t ch3d_resident<float>(int, bool, int*, int*);
+template cudaError_t ch3d_resident<double>(int, bool, int*, int*);
+
 #define GPE2P_CH_INST(R, D)                                                                                 \
   template cudaError_t launch_ch_stage<R, D>(const KParams<R>&, const CHArgs<R>&, int, int, cudaStream_t,   \
                                              const Maps<5>*, int*, const Maps<5>*, const Maps<5>*);        \

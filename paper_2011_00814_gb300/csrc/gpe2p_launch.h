@@ -199,4 +199,8 @@ template <typename real>
 cudaError_t launch_distance(const KParams<real>& P, const real* const f[4], const float* in, int nch, const float* mean,
                             const float* scale, double* part, double* out, cudaStream_t s);
 
+// resident blocks per SM of the 3D CH stage and of mu
+template <typename real>
+cudaError_t ch3d_resident(int iso, bool conservative, int* ch, int* mu);
+
 }  // namespace gpe2p
