@@ -10,7 +10,9 @@
 //               table sweep by sweep and meet at a grid barrier between
 //               sweeps (a bounded wait: after the limit the block records an
 //               error and returns);
-//   per sweep:  one launch per sweep over the whole table.
+//   per sweep:  one launch per sweep over the whole table; in FP32 without
+//               conservative instances the flow stages are one fused pass and the
+//               CH stages with mu another (step2d.cuh).
 // Both are captured into CUDA graphs.  The tile shape and the form are chosen
 // by timing the candidates when the batch is created (the autotuner).  The
 // per-tile arithmetic is the same device code as the single-instance 2D

@@ -1,6 +1,8 @@
 // nn.cu -- kernels of the learned surrogate: a convolutional U-Net on the
 // periodic 2D grid, BF16 activations and weights, FP32 accumulation on the
-// tensor cores (mma.sync m16n8k16), FP32 master weights and Adam.
+// tensor cores, FP32 master weights and Adam.  The 3x3 convolutions and their
+// gradients run on tcgen05 (conv_tc.cu); the warp-level mma.sync forms here are the
+// second backend.
 //
 // Tensors are NHWC: element (b, y, x, c) of a tensor with row stride ldc
 // (channels per pixel, >= the channels used) sits at ((b*H + y)*W + x)*ldc
