@@ -270,8 +270,10 @@ int gpe2p_set_fault_injection(gpe2p_handle h, int what, long long value);
  * conservative advection form (and with the diffusion part of Eq. che in
  * either form); FP32 rounding of phi + dt L makes the integral drift.  With
  * the compensated accumulation on, phi is held as an FP32 high/low pair and
- * the final RK stage of each step forms phi^{n+3/2} in FP64 (about 48
- * significant bits), while the stencils keep reading the FP32 high part.
+ * the final RK stage of each step forms phi^{n+3/2} from that pair and the
+ * FP32 stage increments with every rounding error carried along, so that the
+ * stored pair (about 48 significant bits) is as close to their exact sum as
+ * an FP64 sum rounded to a pair; the stencils keep reading the FP32 high part.
  * Modes: GPE2P_PHI_ACC_FP32 (off), GPE2P_PHI_ACC_COMPENSATED (on),
  * GPE2P_PHI_ACC_AUTO (the default: switched on for the rest of the run at
  * the first diagnostics -- gpe2p_diagnostics, the end of gpe2p_advance and

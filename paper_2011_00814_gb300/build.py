@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libgpe2p.so")
 SOURCES = ["flow.cu", "ch.cu", "diag.cu", "api.cu", "noalloc.cu", "batch.cu", "nn.cu", "net.cu", "pack.cu", "conv_tc.cu", "rate.cu", "step2d.cu"]
-HEADERS = ["gpe2p_dev.cuh", "gpe2p_launch.h", "flow_ops.cuh", "ch_ops.cuh", "ring3d.cuh", "tma.cuh", "batch.h", "nn.h", "step2d.cuh", "diag_ops.cuh"]
+HEADERS = ["gpe2p_dev.cuh", "gpe2p_launch.h", "flow_ops.cuh", "ch_ops.cuh", "ring3d.cuh", "tma.cuh", "batch.h", "nn.h", "step2d.cuh", "diag_ops.cuh", "pair.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-Xptxas", "-warn-spills"]

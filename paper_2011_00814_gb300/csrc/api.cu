@@ -73,7 +73,7 @@ struct gpe2p_ctx {
   double* d_dist = nullptr;     // state-distance scratch (allocated on first use)
   double* h_dist = nullptr;
   // precision policy of the phi accumulation (FP32 problems): low part of phi
-  // when the compensated (FP64) accumulation is on; the mode; the drift
+  // when the compensated accumulation is on; the mode; the drift
   // threshold of the automatic switch and its reference values
   void* phi_lo = nullptr;
   int acc_mode = GPE2P_PHI_ACC_AUTO;

@@ -8,6 +8,7 @@
 #include "flow_ops.cuh"
 #include "gpe2p_dev.cuh"
 #include "gpe2p_launch.h"
+#include "pair.cuh"
 
 namespace gpe2p {
 
@@ -223,40 +224,6 @@ __device__ __forceinline__ real ch_rate(const T& S, const KParams<real>& P, cons
   return -adv + P.M * lapmu;
 }
 
-// The compensated accumulation, phi + lo + (a + d) / 2 or / 6 as a high/low pair, in
-// FP32 pairs: every sum and product that carries rounding (a + d, its sixth,
-// phi plus that) is taken with its error (two-sum, Knuth; the product's by a
-// fused multiply-add, Dekker's product), so what is lost is the rounding of the
-// low parts, about 2^-48 of phi, the precision the pair itself has.  GB300's
-// FP64 pipe is 64 times narrower than its FP32 one: with this sum in FP64 the last
-// CH stage of 101 x 75 x 130 took 42 us, the stages before it 24.
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float t = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
-}
-// ph + (q + qe) + lo, qe and lo small
-__device__ __forceinline__ void pair_sum(float ph, float lo, float q, float qe, float& hi, float& low) {
-  float t, te;
-  two_sum(ph, q, t, te);
-  const float c = __fadd_rn(te, __fadd_rn(lo, qe));
-  hi = __fadd_rn(t, c);
-  low = __fadd_rn(__fsub_rn(t, hi), c);
-}
-__device__ __forceinline__ void pair_half(float ph, float lo, float a, float d, float& hi, float& low) {
-  float s, se;
-  two_sum(a, d, s, se);
-  pair_sum(ph, lo, 0.5f * s, 0.5f * se, hi, low);
-}
-__device__ __forceinline__ void pair_sixth(float ph, float lo, float a, float d, float& hi, float& low) {
-  const float c = (float)(1.0 / 6.0), ce = (float)(1.0 / 6.0 - (double)(float)(1.0 / 6.0));
-  float s, se;
-  two_sum(a, d, s, se);
-  const float q = __fmul_rn(s, c);
-  const float qe = __fadd_rn(__fmaf_rn(s, c, -q), __fmaf_rn(s, ce, __fmul_rn(se, c)));
-  pair_sum(ph, lo, q, qe, hi, low);
-}
-
 // the RK combination of a CH stage for one cell with rate L (phis0 = phi_s
 // at the cell) and its stores; also stores the stage-1 cell velocity
 template <typename real, int DIM>
@@ -268,7 +235,7 @@ __device__ __forceinline__ void ch_finish(const KParams<real>& P, const CHArgs<r
   const bool last = A.stage == A.scheme;
   if (A.phi_lo && last) {
     // phi^{n+3/2} from the high/low pair of phi^{n+1/2} and the stage increments
-    // (never from a rounded stage state), stored back as a pair:
+    // (never from a rounded stage state), stored back as a pair (pair.cuh):
     // RK2 phi^n + (d1 + d2)/2, RK4 phi^n + (d1 + 2 d2 + 2 d3 + d4)/6
     if constexpr (sizeof(real) == 4) {
       real hi, lo;
