@@ -602,6 +602,13 @@ cudaError_t conv3_tc(const ConvArgs& a, cudaStream_t s) {
 // (at most 384 of 512 columns), which then adds them to dW with FP32 reductions
 // coalesced over ci.
 //
+// An accumulator truncates with every K step: sums of terms of one sign lose up to
+// 2^-23 a step.  So a CTA takes at most WG_CHAIN tiles, 2048 pixels, and the chains
+// of a weight meet in FP32 atomics, rounded to nearest.  Error of such a sum
+// (256 -> 256 channels at 128 x 128, batch 8): 4.6e-5 with one chain of 14,600
+// pixels a CTA, 3.6e-6 so; the training step of that net 0.91 and 0.96 ms, of
+// 32-64-128-256 at 256 x 256, whose chains are shorter anyway, 2.02 ms both.
+//
 // Bound: the copies and the MMAs of a tile take nearly the same time beside each
 // other, and the final reductions follow.  All layers of a training step of the
 // 256 x 256, batch 8, 32-64-128-256 net: 0.50 ms (17 launches); without the
@@ -611,6 +618,7 @@ cudaError_t conv3_tc(const ConvArgs& a, cudaStream_t s) {
 constexpr int WG_PROD = 128;              // producer threads (warps 0-3, then the epilogue)
 constexpr int WG_NTHR = WG_PROD + 32;     // warp 4 issues the MMAs
 constexpr int WG_SMAX = 6;
+constexpr int WG_CHAIN = 16;              // tiles a CTA sums in one accumulator, at most
 
 template <int CIB, int COB>
 struct WgCfg {
@@ -815,8 +823,11 @@ cudaError_t launch_wgrad(const ConvArgs& a, cudaStream_t s) {
   const int smem = 1024 + HEAD + ns * C::STAGE;
   const int gy = a.cin / CIB, gz = a.cout / COB;
   long long gx = (long long)occ * nsm / ((long long)gy * gz);
-  if (gx > tiles) gx = tiles;
   if (gx < 1) gx = 1;
+  // chains of at most WG_CHAIN tiles, in whole waves of CTAs
+  const long long chains = (tiles + WG_CHAIN - 1) / WG_CHAIN;
+  if (gx < chains) gx = (chains + gx - 1) / gx * gx;
+  if (gx > tiles) gx = tiles;
   k<<<dim3((unsigned)gx, (unsigned)gy, (unsigned)gz), WG_NTHR, smem, s>>>(a, tiles_x, tiles_y, (int)tiles, ns);
   return cudaGetLastError();
 }
