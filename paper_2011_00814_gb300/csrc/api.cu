@@ -339,7 +339,7 @@ static cudaError_t enqueue_step(gpe2p_ctx* h, int cur, ProfHook* hook = nullptr)
     F.phi = (const float*)h->phi2[cur];
     F.mu = (const float*)h->mu2[cur];
     for (int a = 0; a < 2; ++a) F.usum[a] = usum ? (float*)h->usum[a] : nullptr;
-    if ((e = launch_flow_fused(P, F, s)) != cudaSuccess || (e = mark("flow_step")) != cudaSuccess) return e;
+    if ((e = launch_flow_fused(P, F, false, s)) != cudaSuccess || (e = mark("flow_step")) != cudaSuccess) return e;
     if (h->ch_fused) {
       CHStepArgs<float> G{};
       G.phi = F.phi;
@@ -349,7 +349,7 @@ static cudaError_t enqueue_step(gpe2p_ctx* h, int cur, ProfHook* hook = nullptr)
       G.mu_out = (float*)h->mu2[s1];
       G.lo = (const float*)h->lo2[cur];
       G.lo_out = (float*)h->lo2[s1];
-      if ((e = launch_ch_fused(P, G, s)) != cudaSuccess) return e;
+      if ((e = launch_ch_fused(P, G, false, s)) != cudaSuccess) return e;
       return mark("ch_step");
     }
   } else {
@@ -1012,20 +1012,44 @@ extern "C" int gpe2p_read_fields(gpe2p_handle h, double* phi, double* u, double*
   return GPE2P_OK;
 }
 
+// the rates of the current state by the code that steps it, into Q[2] and phis[1]
+// (phis[0] may hold the other set's phi)
 template <typename real, int DIM>
 static cudaError_t rates_impl(gpe2p_ctx* h) {
   const KParams<real> P = kparams<real>(h->prm);
   const int cur = h->cur;
-  FlowArgs<real> A{};
-  for (int f = 0; f < 4; ++f) {
-    A.q0[f] = (const real*)h->Q[cur][f];
-    A.q[f] = (const real*)h->Q[cur][f];
-    A.out[f] = (real*)h->Q[2][f];
+  cudaError_t e;
+  if constexpr (DIM == 2 && sizeof(real) == 4) {
+    FlowStepArgs<float> F{};
+    for (int f = 0; f < 3; ++f) {
+      F.q[f] = (const float*)h->Q[cur][f];
+      F.out[f] = (float*)h->Q[2][f];
+    }
+    F.phi = (const float*)h->phi;
+    F.mu = (const float*)h->mu;
+    if (h->ch_fused)
+      for (int a = 0; a < 2; ++a) F.usum[a] = (float*)h->usum[a];
+    if ((e = launch_flow_fused(P, F, true, h->stream)) != cudaSuccess) return e;
+    if (h->ch_fused) {
+      CHStepArgs<float> G{};
+      G.phi = F.phi;
+      G.mu = F.mu;
+      for (int a = 0; a < 2; ++a) G.usum[a] = (const float*)h->usum[a];
+      G.phi_out = (float*)h->phis[1];
+      return launch_ch_fused(P, G, true, h->stream);
+    }
+  } else {
+    FlowArgs<real> A{};
+    for (int f = 0; f < 4; ++f) {
+      A.q0[f] = (const real*)h->Q[cur][f];
+      A.q[f] = (const real*)h->Q[cur][f];
+      A.out[f] = (real*)h->Q[2][f];
+    }
+    A.phi = (const real*)h->phi;
+    A.mu = (const real*)h->mu;
+    e = launch_flow_stage<real, DIM>(P, A, 0, h->kchunk, h->stream, &h->flow_maps[cur], h->d_err);
+    if (e != cudaSuccess) return e;
   }
-  A.phi = (const real*)h->phi;
-  A.mu = (const real*)h->mu;
-  cudaError_t e = launch_flow_stage<real, DIM>(P, A, 0, h->kchunk, h->stream, &h->flow_maps[cur], h->d_err);
-  if (e != cudaSuccess) return e;
   CHArgs<real> C{};
   for (int a = 0; a < 3; ++a) {
     C.uh[a] = (real*)h->uh[a];
@@ -1044,7 +1068,7 @@ static cudaError_t rates_impl(gpe2p_ctx* h) {
   C.phis = (const real*)h->phi;
   C.mus = (const real*)h->mu;
   C.phin = (const real*)h->phi;
-  C.out = (real*)h->phis[1];  // (phis[0] may hold the other set's phi)
+  C.out = (real*)h->phis[1];
   return launch_ch_stage<real, DIM>(P, C, h->prm.iso, h->kchunk_ch, h->stream, &h->ch_maps[0], h->d_err);
 }
 

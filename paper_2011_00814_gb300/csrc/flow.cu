@@ -5,7 +5,7 @@
 // u-stress-discretization (a)-(d), st-u-discretization, gradp-u-discretization
 // and gradp-u-p-ave-3d, with phi and mu frozen (Sec. 3, after Eq. tvd-rk3).
 //
-// The operators are in flow_ops.cuh.  2D blocks stage one tile with its halo;
+// The 2D FP64 stage of one tile is in flow_ops.cuh, the 2D FP32 step in step2d.cuh.
 // 3D blocks march along z fed by the TMA plane ring of ring3d.cuh, two cells per
 // thread.
 #include "flow_ops.cuh"
@@ -15,13 +15,7 @@
 
 namespace gpe2p {
 
-// 2D: the FP32 rates (the FP32 step runs in the fused passes of step2d.cuh) and
-// the FP64 stage, one tile per block.
-__global__ void __launch_bounds__(NTHR / 2) rates2d_kernel(const KParams<float> P, const FlowArgs<float> A) {
-  __shared__ float sm2d[F_N * PL];
-  rates2d_tile<float, TX, TY>(P, A, blockIdx.x * TX, blockIdx.y * TY, sm2d);
-}
-
+// 2D FP64: one tile per block (the FP32 step runs in the fused passes of step2d.cuh).
 template <int MODE, int TXv, int TYv, int NT>
 __global__ void __launch_bounds__(NT) flow2d64_kernel(const __grid_constant__ KParams<double> P,
                                                      const FlowArgs<double> A) {
@@ -44,7 +38,7 @@ static cudaError_t flow64_go(const KParams<double>& P, const FlowArgs<double>& A
 // smaller one, since a small grid is bound by the FP64 operations of its
 // busiest SM (64 x 64: 16 tiles of 32 x 8 or 128 of 8 x 4).
 // Measured: 20 steps of 64 x 64 with host arrays in and out 1.73 -> 0.80 ms,
-// 50 steps of 128 x 64 4.05 -> 1.56 ms (32 x 8 tiles of FlowOps before); with
+// 50 steps of 128 x 64 4.05 -> 1.56 ms (32 x 8 tiles with every term formed per cell before); with
 // overlapped launches 0.74 and 1.43 ms.
 static cudaError_t flow64(const KParams<double>& P, const FlowArgs<double>& A, int mode, cudaStream_t s) {
   auto tiles = [&](int tx, int ty) {
@@ -411,15 +405,13 @@ constexpr int flow_ring() { return GPE2P_FLOW_RING; }
 template <typename real, int DIM>
 cudaError_t launch_flow_stage(const KParams<real>& P, const FlowArgs<real>& A, int mode, int kchunk,
                               cudaStream_t s, const Maps<6>* maps, int* err) {
-  dim3 blk(TX, TY, 1);
-  dim3 grd((P.n[0] + TX - 1) / TX, (P.n[1] + TY - 1) / TY, DIM == 3 ? (P.n[2] + kchunk - 1) / kchunk : 1);
-  cudaError_t e;
   if constexpr (DIM == 3) {
     constexpr int RING = flow_ring<real>();
     const size_t sm = 256 + sizeof(real) * (size_t)FlowGeom<real, FLOW_K3_SY>::PE * RING * NRAW_FLOW;
-    blk.y = FLOW_TY;
-    grd.x = (P.n[0] + FLOW_K3_TX - 1) / FLOW_K3_TX;
-    grd.y = (P.n[1] + FLOW_K3_TY - 1) / FLOW_K3_TY;
+    const dim3 blk(TX, FLOW_TY);
+    const dim3 grd((P.n[0] + FLOW_K3_TX - 1) / FLOW_K3_TX, (P.n[1] + FLOW_K3_TY - 1) / FLOW_K3_TY,
+                   (P.n[2] + kchunk - 1) / kchunk);
+    cudaError_t e;
 #define GPE2P_FLOW3_CASE(M)                                                                                 \
   if (P.pavg) {                                                                                             \
     e = cudaFuncSetAttribute(flow3d_kernel<real, M, RING, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
@@ -436,20 +428,15 @@ cudaError_t launch_flow_stage(const KParams<real>& P, const FlowArgs<real>& A, i
     else if (mode == 1) { GPE2P_FLOW3_CASE(1) }
     else { GPE2P_FLOW3_CASE(2) }
 #undef GPE2P_FLOW3_CASE
-  } else if constexpr (sizeof(real) == 8) {
-    return flow64(P, A, mode, s);
+    return cudaGetLastError();
   } else {
-    if (mode != 0) return cudaErrorInvalidValue;  // FP32 steps in fused passes
-    blk.y = TY / 2;  // two cells per thread
-    rates2d_kernel<<<grd, blk, 0, s>>>(P, A);
+    return flow64(P, A, mode, s);
   }
-  return cudaGetLastError();
 }
 
 #define GPE2P_FLOW_INST(R, D)                                                                      \
   template cudaError_t launch_flow_stage<R, D>(const KParams<R>&, const FlowArgs<R>&, int, int, cudaStream_t, \
                                                const Maps<6>*, int*);
-GPE2P_FLOW_INST(float, 2)
 GPE2P_FLOW_INST(float, 3)
 GPE2P_FLOW_INST(double, 2)
 GPE2P_FLOW_INST(double, 3)

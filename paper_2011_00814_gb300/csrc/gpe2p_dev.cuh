@@ -160,22 +160,6 @@ __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(
 __device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
 
-// ---------------------------------------------------------------------------
-// shared-memory tile: NF fields x NPL planes x (SX*SY)
-// ---------------------------------------------------------------------------
-
-template <typename real, int NPL>
-struct Tile {
-  static constexpr int PAVG = -1;  // pressure averaging decided at run time
-  const real* sm;
-  int c;                 // index of the thread's cell within a plane
-  int s0, sm1, sp1;      // plane slots of k, k-1, k+1
-  __device__ __forceinline__ real operator()(int f, int dx, int dy, int dz) const {
-    const int s = dz < 0 ? sm1 : (dz > 0 ? sp1 : s0);
-    return sm[(f * NPL + s) * PL + c + dy * SX + dx];
-  }
-};
-
 __device__ __forceinline__ int clampi(int x, int lo, int hi) { return x < lo ? lo : (x > hi ? hi : x); }
 
 // isotropic lattice weight of the shell |e|^2 = s

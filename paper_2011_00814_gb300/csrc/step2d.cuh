@@ -11,8 +11,8 @@
 // second pass reads phi, mu and the face sums and writes phi and mu: 16 words.
 // The price is a halo of three (flow) or four (CH) cells that neighbouring
 // tiles compute too, 1.4 and 1.5 times the cells at 32 rows.  The arithmetic is
-// that of FlowOps and ch_rate, operation by operation, so the results are the
-// per-stage kernels' bits.
+// the same, operation by operation, in every tile shape and in the batched
+// kernels.
 //
 // A block is NW warps; lane = column, each thread R adjacent rows.  The rows'
 // face and edge terms (normal stresses, corner stresses, diffusive pressure
@@ -157,8 +157,10 @@ struct FlowStepArgs {
 };
 
 // Three flow stages on the tile of FUSED_X x flow_rows(NW R) cells at (i0, j0)
-// by NW warps.  sm: flow_fused_smem reals.
-template <typename real, int NW, int R, bool AXI>
+// by NW warps.  sm: flow_fused_smem reals.  With RATES the first stage alone, its
+// rates L(q) in A.out and u + u in A.usum (the operator-level check runs the code
+// that steps).
+template <typename real, int NW, int R, bool AXI, bool RATES = false>
 __device__ __forceinline__ void flow2d_fused_tile(const KParams<real>& P, const FlowStepArgs<real>& A, int i0, int j0,
                                                   real* sm) {
   constexpr int NR = NW * R, ROWS = NR + 2, PLN = ROWS * 32, NT = 32 * NW;
@@ -278,8 +280,9 @@ __device__ __forceinline__ void flow2d_fused_tile(const KParams<real>& P, const 
   const real half_dx2 = mul_rn(real(0.5), P.inv_dx2);
   const bool wall_tile = (wx && (gi0 < 0 || gi0 + 31 >= nx)) || (wy && (gj0 < 0 || gj0 + ROWS > ny));
 
+  constexpr int NST = RATES ? 1 : 3;
 #pragma unroll
-  for (int st = 1; st <= 3; ++st) {
+  for (int st = 1; st <= NST; ++st) {
     const real* q = st == 1 ? qa : (st == 2 ? qb : qc);
     real* qo = st == 1 ? qb : qc;
     real out[R][3];
@@ -350,6 +353,12 @@ __device__ __forceinline__ void flow2d_fused_tile(const KParams<real>& P, const 
         // faces on a wall are never updated
         if (wx && gi == 0) Lu = real(0);
         if (wy && gj + r == 0) Lv = real(0);
+        if constexpr (RATES) {
+          out[r][0] = Lp;
+          out[r][1] = Lu;
+          out[r][2] = Lv;
+          continue;
+        }
         const real a0 = fma(P.dt, Lp, p[k]), a1 = fma(P.dt, Lu, u[k]), a2 = fma(P.dt, Lv, v[k]);
         if (st == 1) {
           out[r][0] = a0;
@@ -364,7 +373,7 @@ __device__ __forceinline__ void flow2d_fused_tile(const KParams<real>& P, const 
         }
       }
     }
-    if (st < 3) {
+    if (st < NST) {
       // another buffer than any this stage reads (phi and mu are last read
       // before the first barrier of this loop)
       if (live && (!wx || (gi >= 0 && gi < nx))) {
@@ -389,8 +398,9 @@ __device__ __forceinline__ void flow2d_fused_tile(const KParams<real>& P, const 
 #pragma unroll
           for (int f = 0; f < 3; ++f) A.out[f][id] = out[r][f];
           if (A.usum[0]) {
-            A.usum[0][id] = qa[PLN + c0 + 32 * r] + out[r][1];
-            A.usum[1][id] = qa[2 * PLN + c0 + 32 * r] + out[r][2];
+            const real un = qa[PLN + c0 + 32 * r], vn = qa[2 * PLN + c0 + 32 * r];
+            A.usum[0][id] = un + (RATES ? un : out[r][1]);
+            A.usum[1][id] = vn + (RATES ? vn : out[r][2]);
           }
         }
       }
@@ -440,8 +450,9 @@ __device__ __forceinline__ void ch_ghosts(const KParams<real>& P, real* f, int g
 
 // The whole TVD-RK2 CH step of the advective form on the tile of FUSED_X x
 // ch_rows(NW R) cells at (i0, j0): phi_1, mu(phi_1), phi^{n+3/2} and its mu,
-// each on one cell less on every side.  sm: ch_fused_smem reals.
-template <typename real, int NW, int R>
+// each on one cell less on every side.  sm: ch_fused_smem reals.  With RATES the
+// rate of phi alone, in A.phi_out.
+template <typename real, int NW, int R, bool RATES = false>
 __device__ __forceinline__ void ch2d_fused_tile(const KParams<real>& P, const CHStepArgs<real>& A, int i0, int j0,
                                                 real* sm) {
   constexpr int NR = NW * R, ROWS = NR + 2, PLN = ROWS * 34, NT = 32 * NW;
@@ -592,6 +603,16 @@ __device__ __forceinline__ void ch2d_fused_tile(const KParams<real>& P, const CH
     }
   };
   real pn[R], L[R], d1[R], val[R], f1[R];
+  if constexpr (RATES) {
+    if (live) {
+      rate(sa, L, pn);
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        if (lane >= 3 && lane < 3 + FUSED_X && gi < nx && rb + r >= 4 && rb + r < 4 + ch_rows(NR) && gj + r < ny)
+          A.phi_out[(long long)(gj + r) * P.sy + gi] = L[r];
+    }
+    return;
+  }
   if (live) {
     rate(sa, L, pn);
 #pragma unroll
@@ -633,7 +654,8 @@ __device__ __forceinline__ void ch2d_fused_tile(const KParams<real>& P, const CH
   }
 }
 
-cudaError_t launch_flow_fused(const KParams<float>& P, const FlowStepArgs<float>& A, cudaStream_t s);
-cudaError_t launch_ch_fused(const KParams<float>& P, const CHStepArgs<float>& A, cudaStream_t s);
+// the passes of one problem; rates: the rates of the current state in their place
+cudaError_t launch_flow_fused(const KParams<float>& P, const FlowStepArgs<float>& A, bool rates, cudaStream_t s);
+cudaError_t launch_ch_fused(const KParams<float>& P, const CHStepArgs<float>& A, bool rates, cudaStream_t s);
 
 }  // namespace gpe2p
