@@ -45,7 +45,10 @@ GPE2P_HD void two_sum(float a, float b, float& s, float& e) {
   s = r;
 }
 
-// ph + q + the terms y + tail as a pair (tail: terms of third order)
+// ph + q + the terms y + tail as a pair (y: terms of second order, at most half an ulp of
+// ph or q each; tail: of third).  The last sum needs no two-sum: where t is not the
+// larger summand it is what a cancellation left, a multiple of an ulp of ph or
+// q and so of any ulp of s, and the shorter form (Dekker) is exact as well.
 template <int N>
 GPE2P_HD void pair_sum(float ph, float q, const float (&y)[N], float tail, float& hi, float& low) {
   float t, s, e;
@@ -57,8 +60,8 @@ GPE2P_HD void pair_sum(float ph, float q, const float (&y)[N], float tail, float
     two_sum(s, y[i], s, e);
     tail = rn_add(tail, e);
   }
-  two_sum(t, s, hi, e);
-  low = rn_add(e, tail);
+  hi = rn_add(t, s);
+  low = rn_add(rn_add(s, -rn_add(hi, -t)), tail);
 }
 
 // ph + lo + (a + d) / 2
