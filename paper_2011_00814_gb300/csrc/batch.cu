@@ -50,7 +50,7 @@ struct BInst {
   real* phis;      // CH stage state
   real* mus;       // mu of the stage state
   real* uh[2];     // time-centred cell velocity
-  real* z[Z_N];    // FP64: the terms frozen over the flow stages
+  real* z[Z_N];    // FP64: the terms frozen over the flow stages (fill_insts)
   real* us[2];     // u^n + u^{n+1} per face (advective form), left by the last flow stage
   int conservative;
 };
@@ -110,11 +110,11 @@ __device__ __forceinline__ void do_sweep(int sw, const BInst<real>& b, const BIt
     if (sw == SW_FLOW1) {
       A.a = real(0);
       A.b = real(1);
-      if constexpr (sizeof(real) == 8) flow2d_tile64<1, TXv, TYv, TXv * TYv / 2>(b.P, A, it.i0, it.j0, sm);
+      if constexpr (sizeof(real) == 8) flow2d_tile64<1, TXv, TYv, TXv * TYv / 2, false>(b.P, A, it.i0, it.j0, sm);
     } else {
       A.a = sw == SW_FLOW2 ? real(0.75) : real(1.0 / 3.0);
       A.b = sw == SW_FLOW2 ? real(0.25) : real(2.0 / 3.0);
-      if constexpr (sizeof(real) == 8) flow2d_tile64<2, TXv, TYv, TXv * TYv / 2>(b.P, A, it.i0, it.j0, sm);
+      if constexpr (sizeof(real) == 8) flow2d_tile64<2, TXv, TYv, TXv * TYv / 2, false>(b.P, A, it.i0, it.j0, sm);
     }
     return;
   }
@@ -433,7 +433,7 @@ struct BatchCtx {
 };
 
 // field roles inside an instance block
-enum { BF_Q = 0, BF_PHI = 9, BF_MU = 10, BF_PHIS = 11, BF_MUS = 12, BF_UH = 13, BF_US = 15, BF_N = 17, BF_Z = 17 };  // FP64: Z_N more
+enum { BF_Q = 0, BF_PHI = 9, BF_MU = 10, BF_PHIS = 11, BF_MUS = 12, BF_UH = 13, BF_US = 15, BF_N = 17 };
 
 template <typename real>
 static void fill_insts(BatchCtx* b) {
@@ -454,7 +454,20 @@ static void fill_insts(BatchCtx* b) {
     I[k].mu[1] = fld(fused ? BF_MUS : BF_MU);
     I[k].phis = fld(BF_PHIS);
     I[k].mus = fld(BF_MUS);
-    for (int z = 0; z < Z_N; ++z) I[k].z[z] = sizeof(real) == 8 ? fld(BF_Z + z) : nullptr;
+    // FP64: the frozen terms lie in the fields that the flow stages leave free.  The
+    // face sums are written by the last stage, at a face by the thread that has
+    // just read that face's frozen force, and the force alone may lie there.  No
+    // field is left for the corner viscosities: the stages form them anew.
+    static_assert(Z_N == 7, "every frozen term has its place");
+    for (int z = 0; z < Z_N; ++z) I[k].z[z] = nullptr;
+    if (sizeof(real) == 8) {
+      I[k].z[Z_NX] = fld(BF_PHIS);
+      I[k].z[Z_NY] = fld(BF_MUS);
+      I[k].z[Z_RX] = fld(BF_UH);
+      I[k].z[Z_RY] = fld(BF_UH + 1);
+      I[k].z[Z_FX] = fld(BF_US);
+      I[k].z[Z_FY] = fld(BF_US + 1);
+    }
     I[k].uh[0] = fld(BF_UH);
     I[k].uh[1] = fld(BF_UH + 1);
     I[k].us[0] = fld(BF_US);
@@ -739,7 +752,7 @@ int batch_create(const gpe2p_params* p, int n, void* stream, BatchCtx** out, std
     if (p[k].ch_advection) b->any_cons = 1;
     const size_t fb = ((size_t)pitch_of(p[k].nx) * p[k].ny * b->esize + 255) / 256 * 256;
     b->field_off.push_back(off);
-    off += fb * (b->esize == 8 ? BF_N + Z_N : BF_N);
+    off += fb * BF_N;
     b->ncell.push_back((long long)p[k].nx * p[k].ny);
     if (b->ncell.back() > maxcell) maxcell = b->ncell.back();
   }

@@ -71,7 +71,9 @@ __device__ __forceinline__ void stage2d(const KParams<real>& P, int i0, int j0, 
 //     nu, surface tension and gravity, 1 / rho on the faces: all the divisions)
 //     is formed by the first stage (MODE 1) and stored in the fields Z for the
 //     others (MODE 2): 7 words per cell, which stay in L2 or cost less than
-//     the 50 operations they replace;
+//     the 50 operations they replace (without CORNERS, as in a batch, which has
+//     no free field for them, the corner viscosities are formed in every stage:
+//     three additions of staged values, the same bits);
 //   - pressure, u and v of a cell are separate work items, so that a small
 //     tile's chains run side by side.
 // MODE 0: A.out = L(q).  sm: flow64_smem bytes.
@@ -85,7 +87,7 @@ constexpr size_t flow64_smem(int mode) {
   return sizeof(double) * ((size_t)(mode == 2 ? (int)D_PHI : (int)F64_N) * (TXv + 2) * (TYv + 2) + 2 * (TXv + 2));
 }
 
-template <int MODE, int TXv, int TYv, int NT>
+template <int MODE, int TXv, int TYv, int NT, bool CORNERS = true>
 __device__ __forceinline__ void flow2d_tile64(const KParams<double>& P, const FlowArgs<double>& A, int i0, int j0,
                                               double* sm) {
   using real = double;
@@ -152,11 +154,14 @@ __device__ __forceinline__ void flow2d_tile64(const KParams<double>& P, const Fl
       // of the cell up and right: the viscous stress at its low corner, the
       // diffusive pressure fluxes through its low faces
       c += SXv + 1;
+      auto corner4 = [&]() {
+        return (c[D_ETA * PLv] + c[D_ETA * PLv - 1]) + (c[D_ETA * PLv - SXv] + c[D_ETA * PLv - SXv - 1]);
+      };
       real e4, nx2, ny2;
       const int i = i0 + lx, j = j0 + ly;
       if (FROZEN && i < nx && j < ny) {
         const long long id = lin(P, i, j, 0);
-        e4 = A.z[Z_E4][id];
+        e4 = CORNERS ? A.z[Z_E4][id] : corner4();
         nx2 = A.z[Z_NX][id];
         ny2 = A.z[Z_NY][id];
       } else if (FROZEN) {
@@ -166,24 +171,24 @@ __device__ __forceinline__ void flow2d_tile64(const KParams<double>& P, const Fl
         if (wi || wj) {
           // the corner sums of the ghost cells; the flux through a wall is zero
           // (equal pressures on its sides), whatever the viscosity
-          e4 = (c[D_ETA * PLv] + c[D_ETA * PLv - 1]) + (c[D_ETA * PLv - SXv] + c[D_ETA * PLv - SXv - 1]);
+          e4 = corner4();
           const long long id = lin(P, ci == nx ? nx - 1 : ci, cj == ny ? ny - 1 : cj, 0);
           nx2 = A.z[Z_NX][id];
           ny2 = A.z[Z_NY][id];
         } else {
           const long long id = lin(P, ci == nx ? 0 : ci, cj == ny ? 0 : cj, 0);
-          e4 = A.z[Z_E4][id];
+          e4 = CORNERS ? A.z[Z_E4][id] : corner4();
           nx2 = A.z[Z_NX][id];
           ny2 = A.z[Z_NY][id];
         }
       } else {
-        e4 = (c[D_ETA * PLv] + c[D_ETA * PLv - 1]) + (c[D_ETA * PLv - SXv] + c[D_ETA * PLv - SXv - 1]);
+        e4 = corner4();
         const real nu = c[D_NU * PLv];
         nx2 = add_rn(nu, c[D_NU * PLv - 1]);
         ny2 = add_rn(nu, c[D_NU * PLv - SXv]);
         if (MODE == 1 && lx < TXv && ly < TYv && i < nx && j < ny) {
           const long long id = lin(P, i, j, 0);
-          A.z[Z_E4][id] = e4;
+          if (CORNERS) A.z[Z_E4][id] = e4;
           A.z[Z_NX][id] = nx2;
           A.z[Z_NY][id] = ny2;
         }
