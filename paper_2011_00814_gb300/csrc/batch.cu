@@ -18,6 +18,7 @@
 // per-tile arithmetic is the same device code as the single-instance 2D
 // kernels (flow_ops.cuh, ch_ops.cuh), so an instance of a batch follows the
 // single-instance path bit for bit.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -292,21 +293,32 @@ __global__ void __launch_bounds__(32 * NW, ch_blocks(NW, R)) batch_ch_fused_kern
   do_ch_fused<NW, R>(insts[it.inst], it, cur, reinterpret_cast<float*>(smraw));
 }
 
-// the diagnostics of instances k0 .. k0 + gridDim.x / DIAG_NB - 1, DIAG_NB blocks each
-constexpr int DIAG_NB = 32;
-template <typename real>
-__global__ void __launch_bounds__(DIAG_THREADS) batch_diag_kernel(const BInst<real>* __restrict__ insts, int k0, int cur,
-                                                                 double* part) {
-  const int k = k0 + blockIdx.x / DIAG_NB;
+// The diagnostics of instances k0 .. k0 + gridDim.x / nb - 1, nb blocks each: DIAG_NB
+// (a constant: with it as an argument the 96 instances of the batch workload take
+// 403 us in place of 393), or as many as give every SM eight blocks where the
+// instances are few and have 256 cells for each.  The reduction is bound by the
+// FP64 operations of the SMs that take part: one 512 x 512 instance of the 96 takes
+// 64 us with 32 blocks and 50 so, 4096 x 4096 alone in its batch 543 us, as a single
+// problem does.
+constexpr int DIAG_NB = 32, DIAG_FILL = 152 * 8;
+static int diag_blocks(long long count, long long cells) {
+  const long long fill = std::min((DIAG_FILL + count - 1) / count, (cells + DIAG_THREADS - 1) / DIAG_THREADS);
+  return (int)std::max<long long>(DIAG_NB, fill);
+}
+template <typename real, bool FEW>
+__global__ void __launch_bounds__(DIAG_THREADS) batch_diag_kernel(const BInst<real>* __restrict__ insts, int k0, int few_nb,
+                                                                 int cur, double* part) {
+  const int nb = FEW ? few_nb : DIAG_NB;
+  const int k = k0 + blockIdx.x / nb;
   const BInst<real>& b = insts[k];
-  diag_block<real, 2>(b.P, b.Q[cur][0], b.Q[cur][1], b.Q[cur][2], nullptr, b.phi[cur], nullptr, blockIdx.x % DIAG_NB,
-                      DIAG_NB, part + 4 * (size_t)blockIdx.x);
+  diag_block<real, 2>(b.P, b.Q[cur][0], b.Q[cur][1], b.Q[cur][2], nullptr, b.phi[cur], nullptr, blockIdx.x % nb, nb,
+                      part + 4 * (size_t)blockIdx.x);
 }
 template <typename real>
 __global__ void __launch_bounds__(DIAG_THREADS) batch_diag_final_kernel(const BInst<real>* __restrict__ insts, int k0,
-                                                                       const double* part, double* out) {
+                                                                       int nb, const double* part, double* out) {
   const double dx = 1.0 / (double)insts[k0 + blockIdx.x].P.inv_dx;
-  diag_sum(part + 4 * (size_t)blockIdx.x * DIAG_NB, DIAG_NB, dx * dx, out + 4 * (size_t)blockIdx.x);
+  diag_sum(part + 4 * (size_t)blockIdx.x * nb, nb, dx * dx, out + 4 * (size_t)blockIdx.x);
 }
 
 // one sweep SW over the work table, a tile per block: the sweep is a template
@@ -758,7 +770,8 @@ int batch_create(const gpe2p_params* p, int n, void* stream, BatchCtx** out, std
   }
   const size_t state_bytes = off;
   const size_t stage_b = ((size_t)maxcell * sizeof(double) + 255) / 256 * 256;
-  const size_t part_b = ((size_t)n * DIAG_NB * 4 * sizeof(double) + 255) / 256 * 256;
+  const size_t part_n = (size_t)n * DIAG_NB + DIAG_FILL + n;  // of any count up to n
+  const size_t part_b = (part_n * 4 * sizeof(double) + 255) / 256 * 256;
   const size_t out_b = (((size_t)4 * n + 1) * sizeof(double) + 255) / 256 * 256;
   const size_t total = state_bytes + stage_b + part_b + out_b + 256;
   e = cudaMalloc((void**)&b->base, total);
@@ -769,8 +782,9 @@ int batch_create(const gpe2p_params* p, int n, void* stream, BatchCtx** out, std
   }
   b->d_stage = (double*)(b->base + state_bytes);
   b->d_part = (double*)(b->base + state_bytes + stage_b);
-  b->d_out = (double*)(b->base + state_bytes + stage_b + part_b);
-  b->err = (int*)(b->d_out + 4 * (size_t)n);
+  // the error word and after it the results, so that one copy of their length brings both
+  b->err = (int*)(b->base + state_bytes + stage_b + part_b);
+  b->d_out = (double*)b->err + 1;
   b->bar = (BarrierState*)(b->base + state_bytes + stage_b + part_b + out_b);
   if (b->esize == 4) fill_insts<float>(b);
   else fill_insts<double>(b);
@@ -877,12 +891,13 @@ int batch_step(BatchCtx* b, std::string& why) {
 }
 
 template <typename real>
-static cudaError_t batch_diag_impl(BatchCtx* b, int k0, int count) {
+static cudaError_t batch_diag_impl(BatchCtx* b, int k0, int count, int nb) {
   const BInst<real>* insts = (const BInst<real>*)b->insts_dev;
-  batch_diag_kernel<real><<<(unsigned)count * DIAG_NB, DIAG_THREADS, 0, b->stream>>>(insts, k0, b->cur, b->d_part);
+  auto kernel = nb == DIAG_NB ? batch_diag_kernel<real, false> : batch_diag_kernel<real, true>;
+  kernel<<<(unsigned)count * nb, DIAG_THREADS, 0, b->stream>>>(insts, k0, nb, b->cur, b->d_part);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  batch_diag_final_kernel<real><<<(unsigned)count, DIAG_THREADS, 0, b->stream>>>(insts, k0, b->d_part, b->d_out);
+  batch_diag_final_kernel<real><<<(unsigned)count, DIAG_THREADS, 0, b->stream>>>(insts, k0, nb, b->d_part, b->d_out);
   return cudaGetLastError();
 }
 
@@ -894,20 +909,20 @@ int batch_diag(BatchCtx* b, int k, gpe2p_diag* d, std::string& why) {
   gpe2p_diag acc{};
   const int k0 = k < 0 ? 0 : k, count = k < 0 ? b->n : 1;
   if (k >= b->n) { why = "instance index out of range"; return GPE2P_EINVAL; }
-  const size_t all = (size_t)4 * b->n;
-  cudaError_t e = b->esize == 4 ? batch_diag_impl<float>(b, k0, count) : batch_diag_impl<double>(b, k0, count);
+  const int nb = diag_blocks(count, k < 0 ? *std::max_element(b->ncell.begin(), b->ncell.end()) : b->ncell[k]);
+  cudaError_t e = b->esize == 4 ? batch_diag_impl<float>(b, k0, count, nb) : batch_diag_impl<double>(b, k0, count, nb);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(b->h_out, b->d_out, all * sizeof(double) + sizeof(int), cudaMemcpyDeviceToHost, b->stream);
+    e = cudaMemcpyAsync(b->h_out, b->err, (1 + (size_t)4 * count) * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) { why = std::string("diagnostics: ") + cudaGetErrorString(e); return GPE2P_ECUDA; }
   int errw = 0;
-  std::memcpy(&errw, b->h_out + all, sizeof(int));
+  std::memcpy(&errw, b->h_out, sizeof(int));
   if (errw != 0) {
     why = "a grid barrier or device-side copy did not complete within its bounded wait";
     return GPE2P_ETIMEOUT;
   }
   for (int q = 0; q < count; ++q) {
-    const double* o = b->h_out + 4 * (size_t)q;
+    const double* o = b->h_out + 1 + 4 * (size_t)q;
     acc.int_phi += o[0];
     acc.kinetic += o[1];
     acc.umax = o[2] > acc.umax ? o[2] : acc.umax;
