@@ -216,9 +216,11 @@ int gpe2p_field_ptr(gpe2p_handle h, int which, void **dptr, long long *row_pitch
  * gpe2p_advance run every sweep of the method over the tiles of all
  * instances, either as one cooperative persistent launch per step whose
  * blocks meet at a bounded grid barrier between sweeps, or as one launch per
- * sweep; both are captured into CUDA graphs.  The tile shape and the form
- * are chosen at creation by timing each candidate on the zero state (the
- * state is zeroed again afterwards).  gpe2p_diagnostics of a batch sums
+ * sweep; both are captured into CUDA graphs.  (In FP32 the three flow stages
+ * are one sweep, and the CH step of the advective instances another.)  The
+ * form, and the tile shape of the stage-by-stage sweeps (FP64, and the CH step
+ * of conservative instances), are chosen at creation by timing each candidate
+ * on the zero state (the state is zeroed again afterwards).  gpe2p_diagnostics of a batch sums
  * int_phi and kinetic over the instances and takes the max of umax and the
  * NaN flags; gpe2p_init_fields and gpe2p_read_fields do not apply to a batch
  * (GPE2P_EINVAL): use the per-instance calls below. */
@@ -237,8 +239,10 @@ int gpe2p_read_instance(gpe2p_handle h, int inst, double *phi, double *u, double
 /* Diagnostics of one instance of a batch. */
 int gpe2p_diagnostics_instance(gpe2p_handle h, int inst, gpe2p_diag *out);
 
-/* The configuration the autotuner chose for a batch: tile shape, 1 for the
- * persistent form (0: one launch per sweep), and its measured ms per step. */
+/* The configuration of a batch: the tile shape the autotuner chose for the
+ * stage-by-stage sweeps, or the flow sweep's tile if there are none of them
+ * (FP32 without conservative instances); 1 for the persistent form (0: one
+ * launch per sweep), and its measured ms per step. */
 int gpe2p_batch_config(gpe2p_handle h, int *tile_x, int *tile_y, int *persistent, double *ms_per_step);
 
 /* Host-side fault injection and test switches (rebuilds the step graphs).

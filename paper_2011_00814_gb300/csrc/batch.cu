@@ -13,8 +13,9 @@
 //   per sweep:  one launch per sweep over the whole table; in FP32 without
 //               conservative instances the flow stages are one fused pass and the
 //               CH stages with mu another (step2d.cuh).
-// Both are captured into CUDA graphs.  The tile shape and the form are chosen
-// by timing the candidates when the batch is created (the autotuner).  The
+// Both are captured into CUDA graphs.  The form, and the tile shape of the sweeps, are
+// chosen by timing the candidates when the batch is created (the autotuner); the
+// fused passes' tiles by the number of tiles (fused_tall).  The
 // per-tile arithmetic is the same device code as the single-instance 2D
 // kernels (flow_ops.cuh, ch_ops.cuh), so an instance of a batch follows the
 // single-instance path bit for bit.
@@ -935,8 +936,11 @@ int batch_diag(BatchCtx* b, int k, gpe2p_diag* d, std::string& why) {
 }
 
 int batch_config(BatchCtx* b, int* tile_x, int* tile_y, int* persistent, double* ms) {
-  if (tile_x) *tile_x = kShapes[b->shape].tx;
-  if (tile_y) *tile_y = kShapes[b->shape].ty;
+  // without conservative instances an FP32 step is the fused passes alone: the flow pass's tile
+  const bool fused = b->esize == 4 && !b->any_cons;
+  const int rows = b->tall && !b->persistent ? FUSED_NW_TALL * FUSED_R_TALL : FUSED_NW * FUSED_R;
+  if (tile_x) *tile_x = fused ? FUSED_X : kShapes[b->shape].tx;
+  if (tile_y) *tile_y = fused ? flow_rows(rows) : kShapes[b->shape].ty;
   if (persistent) *persistent = b->persistent;
   if (ms) *ms = b->tuned_ms;
   return GPE2P_OK;
