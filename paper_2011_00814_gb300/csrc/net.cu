@@ -367,7 +367,9 @@ extern "C" int gpe2p_net_create(int levels, const int* channels, int in_ch, int 
   n->db.resize(levels);
   if ((e = mk(n->in16, 16, 0))) return fail_alloc(e);
   for (int l = 0; l < levels; ++l) {
-    if ((e = mk(n->ea[l], n->ch[l], l)) || (e = mk(n->eb[l], n->ch[l], l))) return fail_alloc(e);
+    if ((e = mk(n->ea[l], n->ch[l], l))) return fail_alloc(e);
+    // (the other levels' outputs and their gradients live in cat's second half)
+    if (l == levels - 1 && (e = mk(n->eb[l], n->ch[l], l))) return fail_alloc(e);
     if (l < levels - 1) {
       if ((e = mk(n->pooled[l], n->ch[l], l + 1)) || (e = mk(n->upx[l], n->ch[l + 1], l)) ||
           (e = mk(n->cat[l], 2 * n->ch[l], l)) || (e = mk(n->da[l], n->ch[l], l)) || (e = mk(n->db[l], n->ch[l], l)))
