@@ -655,7 +655,9 @@ extern "C" int gpe2p_create(const gpe2p_params* p, void* stream, gpe2p_handle* o
   // from 2, with r blocks resident of the very kernel (3 of the CH stage in FP64
   // conservative form), b blocks on the busiest SM, and the last wave counted by its
   // part of r, at least 0.8 and 0.7 of a wave, since a few blocks do not fill the
-  // SM.  kc is at most 20 and 6, and 4 for the CH stage's ring of five fields in FP32.
+  // SM.  kc is at most 20 and 6, and 4 for the CH stage's ring of five fields in FP32
+  // (there 4 and 20 give the same choice or nearly: six of eight grids the same time,
+  // 101 x 75 x 130 241 and 237 us a step, 80 x 80 x 120 180 and 183).
   // From sweeps of kc over 20 grids.  With the rule above, and with this one, us
   // a step:
   //   FP32                31 x 33 x 40 93, 76   64^3 106, 92   101 x 75 x 130 202, 193

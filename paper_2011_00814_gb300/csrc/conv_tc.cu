@@ -130,13 +130,7 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t v[8]) {
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// z / (1 + exp(-z)); the denominator is at least 1, so the reciprocal needs none
-// of the general quotient's range handling (an infinite one gives zero)
-__device__ __forceinline__ float silu_f(float z) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + __expf(-z)));
-  return z * r;
-}
+__device__ __forceinline__ float silu_f(float z) { return __fdividef(z, 1.0f + __expf(-z)); }
 
 struct TileGeom {
   int b, y0, x0;

@@ -246,7 +246,7 @@ __device__ __forceinline__ void flow2d_fused_tile(const KParams<real>& P, const 
     for (int r = 0; r <= R; ++r) {
       const real sy = et[r + 1] + et[r];  // the column's pair of the corner
       e4u[r] = sy + __shfl_up_sync(FULL, sy, 1);
-      // (add_rn: a plain add could be fused with the quotient's multiply)
+      // (add_rn: rounded by itself in every kernel that inlines this)
       nfy[r] = add_rn(nu[r + 1], nu[r]);
     }
     real sx[R + 1];  // eta(i) + eta(i-1), rows -1 .. R-1
