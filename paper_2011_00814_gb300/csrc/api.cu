@@ -648,8 +648,8 @@ extern "C" int gpe2p_create(const gpe2p_params* p, void* stream, gpe2p_handle* o
   // z-chunks of the marching kernels: a block marches kc planes after a
   // prologue of two, and the blocks run in waves of the resident slots; take
   // the kc in [4, 64] that minimises waves x (kc + 2), the time of the slowest
-  // SM.  Resident blocks per SM (registers and shared memory, as ncu reports
-  // them): flow stage FLOW_MINB, CH stage CH_RESIDENT, mu MU_RESIDENT.
+  // SM.  Blocks per SM reckoned with: flow stage FLOW_MINB, CH stage CH_RESIDENT, mu
+  // MU_RESIDENT (gpe2p_launch.h).
   //
   // CH stage and mu on a grid of at most two waves of marches of four planes: kc
   // from 2, with r blocks resident of the very kernel (3 of the CH stage in FP64

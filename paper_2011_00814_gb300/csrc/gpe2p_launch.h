@@ -65,9 +65,12 @@ constexpr int FLOW_MINB64 = 2;    // FP64: 255 registers a thread, no spills
 constexpr int FLOW_K3_TX = 30;    // columns of a block: the 32 lanes but one on each side
 
 // the blocks of the 3D CH stage and of mu, likewise (2 CH_TY and MU_CPT MU_TY
-// rows of cells), and the blocks of each that fit on an SM: the FP32 CH stage
-// is held by shared memory (its ring and point planes) to nine blocks of four
-// warps, mu by threads to 64 warps.  Four
+// rows of cells), and the blocks of each per SM that the choice of marches on large
+// grids reckons with.  The FP32 CH stage is held to nine blocks of four warps by
+// shared memory (its ring and point planes; stage 1 to eight by its registers).  mu
+// fits 12 at 40 registers, but the marches that the 16 of its threads give are faster:
+// 256 x 256 x 512 2952 us a step, 2958 with 12; 200 x 180 x 220 906 and 910; 128 x 128
+// x 256 and 160^3 the same.  Four
 // warps per CH block measured 0.552 against 0.576 ms for stage 1 (the other
 // stages unchanged).  A mu thread takes MU_CPT = 4 cells in y, so that its
 // plane wait, barrier and addressing serve four cells: 0.094 against 0.114
