@@ -262,11 +262,12 @@ __device__ __forceinline__ void st8(__nv_bfloat16* p, const uint4& v) { *reinter
 // dZ = dY * silu'(z) (dY read with row stride ldy and channel offset yoff) and
 // db[c] += sum over pixels of the stored dZ; a thread takes 8 channels of a
 // pixel, PX pixels at a time so that their loads are in flight together.
-// Bound by HBM (three BF16 tensors) and, with the exact exp and reciprocal,
-// nearly as much by issue.  The channel sums meet by shuffles before one
-// shared-memory add per warp and channel.
-// All 17 layers of a training step at batch 8 (ncu): 460 us one pixel at a time
-// with eight shared adds a thread, 334 us so.
+// Its floor is HBM (three BF16 tensors); what bounds it is issue, with an exp and a
+// quotient per value: 54 % of cycles on the largest layers at three blocks an SM (76
+// registers).  The channel sums meet by shuffles before one shared-memory add per warp
+// and channel.
+// All 17 layers of a training step at batch 8 (ncu): 525 us one pixel at a time
+// with eight shared adds a thread, 450 us so.
 template <int PX>
 __global__ void __launch_bounds__(256) dsilu_bias_kernel(const __nv_bfloat16* dy, int ldy, int yoff,
                                                         const __nv_bfloat16* z, __nv_bfloat16* dz, long long npix, int c,
